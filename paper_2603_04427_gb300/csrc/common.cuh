@@ -90,6 +90,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
   return mbar_wait_for(bar, parity, err, TK_WAIT_LIMIT_NS);
 }
 
+// mbar_wait by a whole warp, the same answer in every lane.  The usual case, a
+// phase that has completed, takes one warp-uniform branch.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, err));
+}
+
 // ---------------------------------------------------------------- dependent launch
 // Kernels launched by launch_pdl may begin while the previous kernel on the
 // stream is still running.  pdl_wait() blocks until that kernel has completed

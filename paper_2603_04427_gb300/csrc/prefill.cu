@@ -33,6 +33,17 @@
 // weights stay <= 256 and the result is unchanged (O / l uses one consistent
 // max).
 //
+// What bounds it: the chain softmax -> P published -> P V -> next scores of each
+// tile (about 2200 cycles per 128 keys and tile pair against 1280 of tensor and
+// 1110 of exponential work), not a pipe.  One warp issues for both tiles because
+// its fixed order A, B keeps the tiles in antiphase: with a warp per tile both
+// softmaxes run, then both wait (7B shape: 754 us a prompt pass against 640).
+// That warp must then be quick: one election per four products and warp-uniform
+// waits.  K and V leave the ring separately (K after its scores, V after its
+// P V products), which a 2-stage ring (r = 128) needs most: B=2, H=32, S=8192,
+// d_v = 128, causal, kernel time before and after both: r=16 625 -> 598 us, r=32
+// 575 -> 563, r=64 617 -> 585, r=128 963 -> 706.
+//
 // TMEM columns: [0,128) S_A, [128,256) S_B (each: fp32 scores, the first 64
 // columns later hold P as packed bf16 pairs), [256,384) O_A, [384,512) O_B.
 #include <algorithm>
@@ -50,9 +61,8 @@ constexpr int kBN = 128;          // keys per kv tile
 constexpr int kThreads = 320;     // 2 x 4 softmax warps, 1 TMA warp, 1 MMA warp
 constexpr int kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
-// P of a tile is published in kParts key ranges, so the P V products of one
-// range run while the softmax computes the next (two halves measured best;
-// four add more handoff latency than they hide).
+// P of a tile is published in kParts key ranges (halves), so the P V products of
+// one range run while the softmax computes the next.
 constexpr int kParts = 2;
 constexpr int kPartPairs = kBN / 2 / kParts;  // packed bf16 pairs (TMEM columns) per part
 
@@ -194,8 +204,9 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   uint64_t* q_full = bars + 0;
   uint64_t* k_full = bars + 1;                  // [NST]
   uint64_t* v_full = k_full + NST;              // [NST]
-  uint64_t* kv_empty = v_full + NST;            // [NST]
-  uint64_t* s_full = kv_empty + NST;            // [2] (tile A, tile B)
+  uint64_t* k_empty = v_full + NST;             // [NST]
+  uint64_t* v_empty = k_empty + NST;            // [NST]
+  uint64_t* s_full = v_empty + NST;             // [2] (tile A, tile B)
   uint64_t* p_full = s_full + 2;                // [tile][part]: P of one key range
   uint64_t* o_full = p_full + 2 * kParts;       // [2]
   uint64_t* c_full = o_full + 2;                // [NST] cached mode: the last tile landed
@@ -242,7 +253,8 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(&k_full[s], 1);
       mbar_init(&v_full[s], 1);
-      mbar_init(&kv_empty[s], 1);
+      mbar_init(&k_empty[s], 1);
+      mbar_init(&v_empty[s], 1);
       mbar_init(&c_full[s], 1);
       mbar_init(&sc_full[s], 1);
     }
@@ -303,12 +315,11 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
           tma_load_3d(smem + C::OFF_Q + x * C::QBA + i * C::QK_BOXB, &maps.q, i * C::QK_BOX,
                       (qa + x) * kBM, bh, q_full);
     }
-    // issue(j): wait for the stage, then the TMA loads of tile j
+    // issue(j): the TMA loads of tile j, K as soon as the scores of the stage's last
+    // tile are computed, V once its P V products are
     auto issue = [&](int j) -> bool {
       const int st = j % NST;
-      int okw = 1;
-      if (j >= NST && lane == 0) okw = mbar_wait(&kv_empty[st], ((j / NST) - 1) & 1, p.err);
-      if (!__shfl_sync(0xffffffffu, okw, 0)) return false;
+      const uint32_t pe = ((j / NST) - 1) & 1;
       // lane s < nsub finds the plane and first row of sub-box s
       int plane = kv_plane, row = j * kBN;
       if (p.page_size != 0) {
@@ -324,43 +335,43 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
         plane = page < 0 ? -1 : page * p.Hkv + g;
         row = t & (p.page_size - 1);
       }
-      int planes[kBN / 16], rows[kBN / 16];
-#pragma unroll
-      for (int s2 = 0; s2 < kBN / 16; ++s2) {
-        planes[s2] = __shfl_sync(0xffffffffu, plane, s2);
-        rows[s2] = __shfl_sync(0xffffffffu, row, s2);
-      }
-      if (lane == 0) {
-        unsigned char* sk = smem + C::OFF_K + st * C::STAGE;
-        unsigned char* sv = sk + C::VOFF;
-        uint64_t* kb = relayed(j) ? &c_full[st] : &k_full[st];
-        if constexpr (KF == kKeyBF16) {
-          mbar_arrive_expect_tx(kb, C::KB);
-          for (int s2 = 0; s2 < nsub; ++s2)
+      if (j >= NST && !mbar_wait_warp(&k_empty[st], pe, p.err)) return false;
+      unsigned char* sk = smem + C::OFF_K + st * C::STAGE;
+      unsigned char* sv = sk + C::VOFF;
+      uint64_t* kb = relayed(j) ? &c_full[st] : &k_full[st];
+      if (lane == 0) mbar_arrive_expect_tx(kb, C::KT * C::KB);
+      if constexpr (KF == kKeyBF16) {
+        for (int s2 = 0; s2 < nsub; ++s2) {
+          const int pl = __shfl_sync(0xffffffffu, plane, s2), rw = __shfl_sync(0xffffffffu, row, s2);
+          if (lane == 0)
             for (int i = 0; i < C::QK_NBOX; ++i)
-              tma_load_3d(sk + i * C::QK_BOXB + s2 * bps * C::QK_SW, &maps.k, i * C::QK_BOX,
-                          rows[s2], planes[s2], kb);
-        } else {
-          // widened keys from the workspace: [B*Hkv][kw_rows][r] planes, one box per tile
-          mbar_arrive_expect_tx(kb, C::KT * C::KB);
-          for (int i = 0; i < C::QK_NBOX; ++i) {
-            tma_load_3d(sk + i * C::QK_BOXB, &maps.k, i * C::QK_BOX, j * kBN, kv_plane, kb);
-            if constexpr (C::KT == 2)
-              tma_load_3d(sk + C::KBA + i * C::QK_BOXB, &maps.klo, i * C::QK_BOX, j * kBN, kv_plane, kb);
-          }
-          if constexpr (C::SCALE_IN_SOFTMAX) {
-            // the tile's key scales (rows past kw_rows are never weighted)
-            const uint32_t bytes = static_cast<uint32_t>(min(kBN, p.kw_rows - j * kBN)) * 4u;
-            mbar_arrive_expect_tx(&sc_full[st], bytes);
-            bulk_g2s(smem + C::OFF_SC + st * C::SCB,
-                     p.kw_scale + static_cast<size_t>(kv_plane) * p.kw_rows + j * kBN, bytes, &sc_full[st]);
-          }
+              tma_load_3d(sk + i * C::QK_BOXB + s2 * bps * C::QK_SW, &maps.k, i * C::QK_BOX, rw, pl, kb);
+        }
+      } else if (lane == 0) {
+        // widened keys from the workspace: [B*Hkv][kw_rows][r] planes, one box per tile
+        for (int i = 0; i < C::QK_NBOX; ++i) {
+          tma_load_3d(sk + i * C::QK_BOXB, &maps.k, i * C::QK_BOX, j * kBN, kv_plane, kb);
+          if constexpr (C::KT == 2)
+            tma_load_3d(sk + C::KBA + i * C::QK_BOXB, &maps.klo, i * C::QK_BOX, j * kBN, kv_plane, kb);
+        }
+      }
+      if (j >= NST && !mbar_wait_warp(&v_empty[st], pe, p.err)) return false;
+      if (lane == 0) {
+        if constexpr (C::SCALE_IN_SOFTMAX) {
+          // the tile's key scales (rows past kw_rows are never weighted); their buffer
+          // is free with V's: the softmax has read them before it publishes P
+          const uint32_t bytes = static_cast<uint32_t>(min(kBN, p.kw_rows - j * kBN)) * 4u;
+          mbar_arrive_expect_tx(&sc_full[st], bytes);
+          bulk_g2s(smem + C::OFF_SC + st * C::SCB,
+                   p.kw_scale + static_cast<size_t>(kv_plane) * p.kw_rows + j * kBN, bytes, &sc_full[st]);
         }
         mbar_arrive_expect_tx(&v_full[st], C::VB);
-        for (int s2 = 0; s2 < nsub; ++s2)
+      }
+      for (int s2 = 0; s2 < nsub; ++s2) {
+        const int pl = __shfl_sync(0xffffffffu, plane, s2), rw = __shfl_sync(0xffffffffu, row, s2);
+        if (lane == 0)
           for (int i = 0; i < C::V_NBOX; ++i)
-            tma_load_3d(sv + i * C::V_BOXB + s2 * bps * 128, &maps.v, i * 64, rows[s2], planes[s2],
-                        &v_full[st]);
+            tma_load_3d(sv + i * C::V_BOXB + s2 * bps * 128, &maps.v, i * 64, rw, pl, &v_full[st]);
       }
       return true;
     };
@@ -393,35 +404,31 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
         tc_commit_e(&s_full[x]);
       };
       auto issue_pv = [&](int x, int st, bool first, int part) {  // O_x += P_x V, one part
-        const uint32_t vo = st * C::STAGE;
-        const uint32_t td = tmem + 256 + x * 128, ta = tmem + x * 128;
-#pragma unroll
-        for (int kk = 0; kk < kBN / 16 / kParts; ++kk) {
-          const int k = part * (kBN / 16 / kParts) + kk;
-          mma_ts_e(td, ta + 8 * k, dv.at(vo + k * 16 * 128), C::IDESC_O, (!first || k > 0) ? 1u : 0u);
-        }
+        static_assert(kBN / 16 / kParts == 4, "four K steps per part");
+        mma_ts4_e(tmem + 256 + x * 128, tmem + x * 128 + 32 * part, dv.at(st * C::STAGE + part * (64 * 128)),
+                  16 * 128, C::IDESC_O, (first && part == 0) ? 0u : 1u);
       };
-      bool ok = __all_sync(0xffffffffu, mbar_wait(q_full, 0, p.err) && mbar_wait(&k_full[0], 0, p.err));
+      bool ok = mbar_wait_warp(q_full, 0, p.err) && mbar_wait_warp(&k_full[0], 0, p.err);
       if (ok) {
         tc_fence_after();
         issue_s(0, 0);
         if (has_b) issue_s(1, 0);
+        tc_commit_e(&k_empty[0]);
       }
       for (int j = 0; ok && j < n_kv; ++j) {
         const int st = j % NST;
-        const uint32_t ph = (j / NST) & 1;
         const int stn = (j + 1) % NST;
-        const uint32_t phn = ((j + 1) / NST) & 1;
-        bool v_ready = false;
+        if (!(ok = mbar_wait_warp(&v_full[st], (j / NST) & 1, p.err))) break;
+        bool k_ready = false;
         for (int x = 0; x < 2 && ok; ++x) {
           const int nx = x == 0 ? n_a : n_b;
           if (j >= nx) continue;
           // each part of P_x(j) feeds its MMAs while the softmax warps compute
           // the next part
-          if (!v_ready && !(ok = __all_sync(0xffffffffu, mbar_wait(&v_full[st], ph, p.err)))) break;
-          v_ready = true;
-          for (int h = 0; ok && h < kParts; ++h) {
-            if (!(ok = __all_sync(0xffffffffu, mbar_wait(&p_full[kParts * x + h], j & 1, p.err)))) break;
+#pragma unroll
+          for (int h = 0; h < kParts; ++h) {
+            if (ok) ok = mbar_wait_warp(&p_full[kParts * x + h], j & 1, p.err);
+            if (!ok) break;
             tc_fence_after();
             issue_pv(x, st, j == 0, h);
           }
@@ -429,12 +436,15 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
           if (j + 1 == nx) {
             tc_commit_e(&o_full[x]);
           } else {
-            if (!(ok = __all_sync(0xffffffffu, mbar_wait(&k_full[stn], phn, p.err)))) break;
+            if (!k_ready && !(ok = mbar_wait_warp(&k_full[stn], ((j + 1) / NST) & 1, p.err))) break;
+            k_ready = true;
             tc_fence_after();
             issue_s(x, stn);
           }
         }
-        if (ok) tc_commit_e(&kv_empty[st]);
+        if (!ok) break;
+        if (j + 1 < n_kv) tc_commit_e(&k_empty[stn]);
+        tc_commit_e(&v_empty[st]);
       }
     }
   } else {
