@@ -3,13 +3,17 @@
 Argument marshalling only: each function checks that the torch tensors it
 is given have the dtype, device and contiguity the C ABI expects, passes
 their ``data_ptr()`` and the current CUDA stream, and raises ``TkError`` on
-a non-OK status.  Every step of the computation runs in the library's
+a non-OK status.  The hot functions first offer their arguments to the native
+module (csrc/py_binding.cpp), which makes the same checks and the C call and
+returns its status, or None if an argument is not the plain case: then the
+checks here raise what is wrong or marshal the rest.  Every step of the computation runs in the library's
 kernels; there is no CPU or PyTorch fallback, and a missing library raises.
 """
 
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import math
 import os
 from dataclasses import dataclass
@@ -42,7 +46,12 @@ class tk_cache_desc(ctypes.Structure):
         "max_pages_per_seq", "k_dtype")]
 
 
+NATIVE_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tkpy.so")
+_NATIVE_CALLS = ("tk_kv_append", "tk_attn_decode", "tk_attn_decode_append", "tk_attn_decode_noalloc",
+                 "tk_attn_prefill", "tk_attn_forward", "tk_attn_backward", "tk_attn_prefill_cached")
+
 _lib = None
+_native = None
 
 
 def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
@@ -86,8 +95,28 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
+    _load_native(L)
     _lib = L
     return L
+
+
+def _load_native(L: ctypes.CDLL):
+    """Load _tkpy.so and give it the addresses of the library's entry points."""
+    global _native
+    if not os.path.exists(NATIVE_PATH):
+        raise RuntimeError(f"{NATIVE_PATH} is not built; run `python -m paper_2603_04427_gb300.build` "
+                           "(or __graft_entry__.build()) first")
+    spec = importlib.util.spec_from_file_location(f"{__package__}._tkpy", NATIVE_PATH)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.bind(*(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _NATIVE_CALLS))
+    _native = m
+
+
+def _fast():
+    if _native is None:
+        load_library()
+    return _native
 
 
 def _status_name(s: int) -> str:
@@ -190,6 +219,11 @@ def tk_last_error() -> str:
 
 def tk_kv_append(cache: ThinKeyCache, k_new, v_new, seq_lens, stream=None):
     """Append k_new [B, H_kv, T, r] / v_new [B, H_kv, T, d_v] (bf16) at seq_lens[b]."""
+    st = _fast().kv_append(cache, k_new, v_new, seq_lens, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_kv_append")
+        return
     d = cache.desc
     dev = cache.k.device
     _need(k_new, torch.bfloat16, "k_new", dev)
@@ -220,6 +254,11 @@ def tk_attn_decode(cache: ThinKeyCache, q, seq_lens, max_seq_len: int, out, work
                    scale: float | None = None, stream=None):
     """One decode step: q [B, H_q, r] bf16 -> out [B, H_q, d_v] (fp32 or bf16, on the GPU or
     in page-locked host memory, which the kernel then writes directly)."""
+    st = _fast().decode(cache, q, seq_lens, max_seq_len, out, workspace, scale, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_decode")
+        return out
     d = cache.desc
     dev = cache.k.device
     _need(q, torch.bfloat16, "q", dev)
@@ -242,6 +281,12 @@ def tk_attn_decode_append(cache: ThinKeyCache, q, k_new, v_new, seq_lens, max_se
                           workspace, scale: float | None = None, stream=None):
     """Append one token per sequence (k_new [B, H_kv, r], v_new [B, H_kv, d_v] bf16) at
     seq_lens[b] and decode q [B, H_q, r] over the seq_lens[b] + 1 tokens, in one launch."""
+    st = _fast().decode_append(cache, q, k_new, v_new, seq_lens, max_seq_len, out, workspace,
+                               scale, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_decode_append")
+        return out
     d = cache.desc
     dev = cache.k.device
     _need(q, torch.bfloat16, "q", dev)
@@ -267,6 +312,11 @@ def tk_attn_decode_append(cache: ThinKeyCache, q, k_new, v_new, seq_lens, max_se
 
 def tk_attn_forward(q, k, v, out, lse, scale: float | None = None, causal: bool = True, stream=None):
     """tk_attn_prefill that also writes lse [B, H_q, S] (fp32), each row's logsumexp."""
+    st = _fast().forward(q, k, v, out, lse, scale, causal, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_forward")
+        return out, lse
     dev = q.device
     for t, n in ((q, "q"), (k, "k"), (v, "v")):
         _need(t, torch.bfloat16, n, dev)
@@ -292,6 +342,11 @@ def tk_attn_backward(q, k, v, out, d_out, lse, dq, dk, dv, workspace=None,
                      scale: float | None = None, causal: bool = True, stream=None):
     """Gradients dq [B, H_q, S, r], dk [B, H_kv, S, r], dv [B, H_kv, S, d_v] (fp32)
     of prefill attention for dL/d(out) = d_out (bf16), from the forward's lse."""
+    st = _fast().backward(q, k, v, out, d_out, lse, dq, dk, dv, workspace, scale, causal, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_backward")
+        return dq, dk, dv
     dev = q.device
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (out, "out"), (d_out, "d_out")):
         _need(t, torch.bfloat16, n, dev)
@@ -331,6 +386,12 @@ def tk_attn_prefill_cached(cache: ThinKeyCache, q, k_new, v_new, seq_lens, max_s
     and prefill its queries q [B, H_q, S, r] over the cache (query i at position
     seq_lens[b] + i) -> out [B, H_q, S, d_v] (fp32 or bf16).  bf16, int8 or int4 keys;
     quantised keys need a workspace (prefill_cached_workspace; allocated here if None)."""
+    st = _fast().prefill_cached(cache, q, k_new, v_new, seq_lens, max_seq_len, out, scale, causal,
+                                workspace, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_prefill_cached")
+        return out
     d = cache.desc
     dev = cache.k.device
     for t, n in ((q, "q"), (k_new, "k_new"), (v_new, "v_new")):
@@ -474,6 +535,11 @@ def prepare_decode_append(cache: ThinKeyCache, q, k_new, v_new, seq_lens, max_se
 
 def tk_attn_prefill(q, k, v, out, scale: float | None = None, causal: bool = True, stream=None):
     """Prefill: q [B, H_q, S, r], k [B, H_kv, S, r], v [B, H_kv, S, d_v] bf16 -> out [B, H_q, S, d_v]."""
+    st = _fast().prefill(q, k, v, out, scale, causal, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_prefill")
+        return out
     dev = q.device
     for t, n in ((q, "q"), (k, "k"), (v, "v")):
         _need(t, torch.bfloat16, n, dev)
@@ -501,6 +567,11 @@ def tk_attn_decode_noalloc(cache: ThinKeyCache, q, seq_lens, max_seq_len: int, o
     For callers that cannot allocate device memory.  Calls that may overlap on
     the GPU share the scratch and race; see include/tk.h.
     """
+    st = _fast().decode_noalloc(cache, q, seq_lens, max_seq_len, out, scale, stream)
+    if st is not None:
+        if st != TK_OK:
+            _check(st, "tk_attn_decode_noalloc")
+        return out
     d = cache.desc
     dev = cache.k.device
     _need(q, torch.bfloat16, "q", dev)

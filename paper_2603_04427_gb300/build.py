@@ -1,8 +1,9 @@
 """Build ``libtk.so`` (the CUDA library behind include/tk.h) in-tree for sm_103a.
 
 Each ``csrc/*.cu`` is compiled by nvcc in parallel, then linked into
-``paper_2603_04427_gb300/libtk.so``.  The build is skipped when the library
-is newer than every source and header.  Run ``python -m
+``paper_2603_04427_gb300/libtk.so``; ``csrc/py_binding.cpp`` (the binding's
+native argument checks) is compiled by g++ beside them into ``_tkpy.so``.  The
+build is skipped when both are newer than every source and header.  Run ``python -m
 paper_2603_04427_gb300.build`` (or ``__graft_entry__.build()``).
 """
 
@@ -14,6 +15,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -21,6 +23,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtk.so")
+PY_SRC = os.path.join(CSRC, "py_binding.cpp")
+PY_LIB = os.path.join(PKG, "_tkpy.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
@@ -39,14 +43,14 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
+    return _sources() + [PY_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
         os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PY_LIB):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_LIB))
     return all(os.path.getmtime(f) <= t for f in _deps() + [__file__])
 
 
@@ -61,6 +65,25 @@ def _compile(src: str, extra) -> str:
     return obj
 
 
+def _build_py() -> None:
+    """_tkpy.so: a CPython module over torch's C++ tensors (paths of the installed torch)."""
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(os.path.abspath(nvcc())))
+    inc = [sysconfig.get_paths()["include"], os.path.join(root, "include"),
+           os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), INCLUDE]
+    tmp = PY_LIB + ".tmp"
+    cmd = (["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+           + [x for d in inc for x in ("-isystem", d)] + [PY_SRC, "-o", tmp, "-L", os.path.join(root, "lib"),
+              "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"])
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for {PY_SRC}:\n{' '.join(cmd)}\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, PY_LIB)
+
+
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     """Compile and link libtk.so; returns its path."""
     if not force and up_to_date():
@@ -68,8 +91,10 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
     os.makedirs(BUILD, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose_ptxas else []
     srcs = _sources()
-    with cf.ThreadPoolExecutor(max_workers=max(1, min(len(srcs), os.cpu_count() or 1))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=max(1, min(len(srcs) + 1, os.cpu_count() or 1))) as ex:
+        py = ex.submit(_build_py)
         objs = list(ex.map(lambda s: _compile(s, extra), srcs))
+    py.result()
     tmp = LIB + ".tmp"
     cmd = [nvcc()] + ARCH + ["-shared", "-o", tmp] + objs
     r = subprocess.run(cmd, capture_output=True, text=True)
