@@ -30,6 +30,8 @@ __global__ void __launch_bounds__(kPrepThreads) bwd_prep(const BackwardParams p)
   constexpr int TPR = DV / 8;                       // threads per row
   constexpr int RPB = kPrepThreads / TPR;           // rows per block
   static_assert(32 % TPR == 0, "a row's threads sit in one warp");
+  pdl_wait();
+  pdl_trigger();
   const int sub = threadIdx.x % TPR;
   const long long row = static_cast<long long>(blockIdx.x) * RPB + threadIdx.x / TPR;
   const long long rows = static_cast<long long>(p.B) * p.Hq * p.S_pad;
@@ -66,8 +68,8 @@ cudaError_t launch_t(const BackwardParams& p, cudaStream_t s, int* uns) {
   constexpr int rpb = kPrepThreads / (DV / 8);
   const long long pblocks = (rows + rpb - 1) / rpb;
   if (pblocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  bwd_prep<R, DV><<<static_cast<unsigned>(pblocks), kPrepThreads, 0, s>>>(p);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_pdl(bwd_prep<R, DV>, dim3(static_cast<unsigned>(pblocks)), dim3(kPrepThreads), 0, s, p);
   if (e != cudaSuccess) return e;
   return launch_backward_tc(p, s, uns);
 }

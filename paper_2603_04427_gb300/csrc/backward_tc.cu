@@ -264,7 +264,18 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     tmem_alloc(tmem_slot, kTmemColsTc);
     tmem_relinquish();
   }
+  if (warp == 9 && lane == 0) {
+    prefetch_map(&maps.q);
+    prefetch_map(&maps.k);
+    prefetch_map(&maps.v);
+    prefetch_map(&maps.d_out);
+  }
+  // the set-up above reads no global memory: it runs while the previous kernel finishes
+  pdl_wait();
   __syncthreads();
+  // after the barrier, so that every CTA of this grid holds its TMEM before a
+  // CTA of the next kernel can ask for some
+  pdl_trigger();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -272,10 +283,6 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const int kv_plane = b * p.Hkv + g;
-      prefetch_map(&maps.q);
-      prefetch_map(&maps.k);
-      prefetch_map(&maps.v);
-      prefetch_map(&maps.d_out);
       mbar_arrive_expect_tx(kv_full, C::KB + C::VB);
       for (int x = 0; x < C::QK_NBOX; ++x)
         tma_load_3d(smem + C::OFF_K + x * C::KBOX, &maps.k, x * C::QK_BOXW, j * kKeys, kv_plane, kv_full);
@@ -629,8 +636,7 @@ cudaError_t launch_tc(const BackwardParams& p, cudaStream_t stream) {
   const long long n_kt = (p.S + kKeys - 1) / kKeys;
   const long long grid = static_cast<long long>(p.B) * p.Hkv * n_kt;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  kern<<<static_cast<unsigned>(grid), kTcThreads, C::SMEM, stream>>>(maps, p);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(kTcThreads), C::SMEM, stream, maps, p);
 }
 
 template <int R>

@@ -228,6 +228,34 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   const int kv_plane = b * p.Hkv + h / (p.Hq / p.Hkv);
   const int qa = 2 * tp, qb = 2 * tp + 1;
   const bool has_b = qb < n_qt;
+  // set-up that reads no global memory runs while the previous kernel finishes
+  if (tid == 0) {
+    mbar_init(q_full, 1);
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&k_full[s], 1);
+      mbar_init(&v_full[s], 1);
+      mbar_init(&k_empty[s], 1);
+      mbar_init(&v_empty[s], 1);
+      mbar_init(&c_full[s], 1);
+      mbar_init(&sc_full[s], 1);
+    }
+    for (int x = 0; x < 2; ++x) {
+      mbar_init(&s_full[x], 1);
+      for (int h = 0; h < kParts; ++h) mbar_init(&p_full[kParts * x + h], 128);
+      mbar_init(&o_full[x], 1);
+    }
+    fence_barrier_init();
+  }
+  if (warp == 8) {
+    if (lane == 0) {
+      prefetch_map(&maps.q);
+      prefetch_map(&maps.k);
+      prefetch_map(&maps.v);
+    }
+    tmem_alloc(tmem_slot, kTmemCols);
+    tmem_relinquish();
+  }
+  pdl_wait();
   // keys: the sequence's first kv_len cache tokens; query row i sits at position L0 + i
   int L0 = 0;
   if (p.seq_lens) {
@@ -248,28 +276,10 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   const int n_b = has_b ? tiles_for(qb) : 0;
   const int n_kv = max(n_a, n_b);
 
-  if (tid == 0) {
-    mbar_init(q_full, 1);
-    for (int s = 0; s < NST; ++s) {
-      mbar_init(&k_full[s], 1);
-      mbar_init(&v_full[s], 1);
-      mbar_init(&k_empty[s], 1);
-      mbar_init(&v_empty[s], 1);
-      mbar_init(&c_full[s], 1);
-      mbar_init(&sc_full[s], 1);
-    }
-    for (int x = 0; x < 2; ++x) {
-      mbar_init(&s_full[x], 1);
-      for (int h = 0; h < kParts; ++h) mbar_init(&p_full[kParts * x + h], 128);
-      mbar_init(&o_full[x], 1);
-    }
-    fence_barrier_init();
-  }
-  if (warp == 8) {
-    tmem_alloc(tmem_slot, kTmemCols);
-    tmem_relinquish();
-  }
   __syncthreads();
+  // after the barrier, so that every CTA of this grid holds its TMEM before a
+  // CTA of the next kernel can ask for some
+  pdl_trigger();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -306,9 +316,6 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     const int bps = (p.page_size == 0 || p.page_size >= kBN) ? kBN : p.page_size;
     const int nsub = kBN / bps;
     if (lane == 0) {
-      prefetch_map(&maps.q);
-      prefetch_map(&maps.k);
-      prefetch_map(&maps.v);
       mbar_arrive_expect_tx(q_full, has_b ? 2 * C::QB : C::QB);
       for (int x = 0; x < (has_b ? 2 : 1); ++x)
         for (int i = 0; i < C::QK_NBOX; ++i)
@@ -617,6 +624,8 @@ template <int R, int KF, int KT>
 __global__ void __launch_bounds__(256) key_widen_kernel(const PrefillParams p, __nv_bfloat16* hi,
                                                         __nv_bfloat16* lo, float* sc) {
   constexpr int PPR = R / 8;
+  pdl_wait();
+  pdl_trigger();
   const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= static_cast<long long>(p.B) * p.Hkv * p.kw_rows * PPR) return;
   const int piece = static_cast<int>(i % PPR);
@@ -722,14 +731,14 @@ cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   if (grid > 0x7fffffffL) return cudaErrorInvalidConfiguration;
   if constexpr (KF != kKeyBF16) {
     const long long n = static_cast<long long>(p.B) * p.Hkv * p.kw_rows * (R / 8);
-    key_widen_kernel<R, KF, C::KT><<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(p, hi, lo, sc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_pdl(key_widen_kernel<R, KF, C::KT>, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, stream,
+                   p, hi, lo, sc);
+    if (e != cudaSuccess) return e;
   }
   // about 48 MB of K/V per head group
   const long head_bytes = static_cast<long>(p.seq_lens ? p.kv_limit : p.S) * (R + DV) * 2;
   pp.head_group = static_cast<int>(std::max(1L, std::min<long>(p.B * p.Hq, (48L << 20) / head_bytes)));
-  kern<<<static_cast<unsigned>(grid), kThreads, smem, stream>>>(maps, pp);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem, stream, maps, pp);
 }
 
 template <int R, int DV>
