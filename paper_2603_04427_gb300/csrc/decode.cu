@@ -52,6 +52,7 @@ namespace {
 constexpr int kChunk = 64;                  // tokens per unit / pipeline stage
 constexpr int kCW = 4;                      // consumer warps (16 tokens each)
 constexpr int kThreads = (kCW + 2) * 32;    // + one producer warp + one merger warp
+constexpr int kMaxSub = 4;                  // pages of 16 tokens in one unit
 constexpr int kMaxBatch = 1024;             // prefix arrays live in shared memory
 constexpr int kCtaSmemTarget = 110 * 1024;  // aim for two CTAs per SM
 
@@ -388,27 +389,33 @@ __device__ void prefetch_first_chunks(const DecodeParams& p, int lane, int limit
   if (lane >= nunits || u >= u_end || nb == 0) return;
   const long long off = u - pb;
   const int g = static_cast<int>(off / nb), t0 = static_cast<int>(off % nb) * kChunk;
-  long long row;
-  int rows;
+  auto fetch = [&](long long row, int rows) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const unsigned char*>(p.k) + row * RB),
+                 "r"(static_cast<uint32_t>(rows * RB))
+                 : "memory");
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const unsigned char*>(p.v) + row * DV * 2),
+                 "r"(static_cast<uint32_t>(rows * DV * 2))
+                 : "memory");
+  };
   if (p.page_size == 0) {
-    row = (static_cast<long long>(b) * Hkv + g) * p.capacity + t0;
-    rows = min(kChunk, p.capacity - t0);
+    const int rows = min(kChunk, p.capacity - t0);
+    if (rows > 0) fetch((static_cast<long long>(b) * Hkv + g) * p.capacity + t0, rows);
   } else {
-    const int pidx = t0 >> p.page_shift;
-    if (pidx >= p.max_pages) return;
-    const int page = p.page_table[static_cast<long long>(b) * p.max_pages + pidx];
-    if (page < 0 || page >= p.num_pages) return;
-    const int in_page = t0 & (p.page_size - 1);
-    row = (static_cast<long long>(page) * Hkv + g) * p.page_size + in_page;
-    rows = min(kChunk, p.page_size - in_page);
+    // the chunk's part of one page, or its 64 / page_size pages
+    const int in_page = t0 & (p.page_size - 1), rows = min(kChunk, p.page_size - in_page);
+    int page[kMaxSub];
+#pragma unroll
+    for (int s = 0; s < kMaxSub; ++s) {
+      const int t = t0 + s * rows, pidx = t >> p.page_shift;
+      page[s] = s * rows < kChunk && t < Lb && pidx < p.max_pages
+                    ? p.page_table[static_cast<long long>(b) * p.max_pages + pidx]
+                    : -1;
+    }
+#pragma unroll
+    for (int s = 0; s < kMaxSub; ++s)
+      if (page[s] >= 0 && page[s] < p.num_pages)
+        fetch((static_cast<long long>(page[s]) * Hkv + g) * p.page_size + in_page, rows);
   }
-  if (rows <= 0) return;
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const unsigned char*>(p.k) + row * RB),
-               "r"(static_cast<uint32_t>(rows * RB))
-               : "memory");
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const unsigned char*>(p.v) + row * DV * 2),
-               "r"(static_cast<uint32_t>(rows * DV * 2))
-               : "memory");
 }
 
 
@@ -502,7 +509,8 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     bool ok = true;
     for (long long w0 = u_begin; ok && w0 < u_end; w0 += 32) {
       // lane j prepares unit w0 + j: first cache row of the chunk, valid tokens, query offset
-      long long row = 0, app = -1;
+      long long app = -1;
+      int row[kMaxSub] = {};  // of each box of the chunk (one, or one per page of 16 or 32 tokens)
       int n = 0, qoff = 0, g = 0, b = 0, t0 = 0;
       const long long u = w0 + lane;
       if (u < u_end) {
@@ -529,24 +537,36 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
           }
         }
         if (ps == 0) {
-          row = (static_cast<long long>(b) * Hkv + g) * p.capacity + t0;
+          row[0] = (b * Hkv + g) * p.capacity + t0;  // rows are below 2^31 (checked on the host)
         } else {
-          int page = p.page_table[static_cast<long long>(b) * p.max_pages + (t0 >> p.page_shift)];
-          if (page < 0 || page >= p.num_pages) {
-            record_error(p.err, TK_DEVERR_INDEX);
-            page = 0;
+          // all page ids of the chunk in one round of loads; boxes past the
+          // context are not loaded (a warp's 16 rows are one box or part of one)
+          int page[kMaxSub];
+#pragma unroll
+          for (int s = 0; s < kMaxSub; ++s) {
+            page[s] = 0;
+            if (s == 0 || s * rows_per_box < n)
+              page[s] = p.page_table[static_cast<long long>(b) * p.max_pages + ((t0 + s * rows_per_box) >> p.page_shift)];
           }
-          row = (static_cast<long long>(page) * Hkv + g) * ps + (t0 & (ps - 1));
+#pragma unroll
+          for (int s = 0; s < kMaxSub; ++s) {
+            if (page[s] < 0 || page[s] >= p.num_pages) {
+              record_error(p.err, TK_DEVERR_INDEX);
+              page[s] = 0;
+            }
+            row[s] = (page[s] * Hkv + g) * ps + (s == 0 ? t0 & (ps - 1) : 0);
+          }
         }
       }
       const int cnt = static_cast<int>(min(32LL, u_end - w0));
       for (int j = 0; j < cnt; ++j) {
-        const long long rj = __shfl_sync(0xffffffffu, row, j);
+        int rj[kMaxSub];
+#pragma unroll
+        for (int s = 0; s < kMaxSub; ++s) rj[s] = __shfl_sync(0xffffffffu, row[s], j);
         const int nj = __shfl_sync(0xffffffffu, n, j);
         const int qj = __shfl_sync(0xffffffffu, qoff, j);
         const int bj = __shfl_sync(0xffffffffu, b, j);
         const int gj = __shfl_sync(0xffffffffu, g, j);
-        const int tj = __shfl_sync(0xffffffffu, t0, j);
         const long long aj = __shfl_sync(0xffffffffu, app, j);
         if (aj >= 0) {
           // the new row, then a proxy fence: the TMA reads below see it
@@ -566,29 +586,24 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
           if (ok) {
             unsigned char* sk = smem + st * C::STAGE;
             const uint32_t sbytes = KI8 ? ((nj + 3) & ~3) * 4 : 0;
-            mbar_arrive_expect_tx(&full[st], C::KB + C::VB + sbytes + C::QB);
-            // rows_per_box = 64 except for pages of 16 or 32 tokens
-            for (int t = 0; t < kChunk; t += rows_per_box) {
-              long long r2 = rj + t;
-              if (t > 0 && ps != 0) {
-                const int pidx = (tj + t) >> p.page_shift;
-                // pages past the context are never read back: any valid page will do
-                int page = pidx < p.max_pages ? p.page_table[static_cast<long long>(bj) * p.max_pages + pidx] : 0;
-                if (page < 0 || page >= p.num_pages) page = 0;
-                r2 = (static_cast<long long>(page) * Hkv + gj) * ps;
-              }
+            // rows_per_box = 64 except for pages of 16 or 32 tokens; nj >= 1
+            const int boxes = (nj + rows_per_box - 1) / rows_per_box;
+            mbar_arrive_expect_tx(&full[st], boxes * rows_per_box * ((C::KB + C::VB) / kChunk) + sbytes + C::QB);
+#pragma unroll
+            for (int s = 0; s < kMaxSub; ++s) {
+              if (s >= boxes) break;
+              const int t = s * rows_per_box;
 #pragma unroll
               for (int kb = 0; kb < C::KBOX_N; ++kb)
-                tma_load_2d(sk + kb * C::KBOX + t * C::KSW, &maps.k, kb * (C::KSW / (KI8 ? 1 : 2)),
-                            static_cast<int>(r2), &full[st], pol);
+                tma_load_2d(sk + kb * C::KBOX + t * C::KSW, &maps.k, kb * (C::KSW / (KI8 ? 1 : 2)), rj[s], &full[st],
+                            pol);
 #pragma unroll
               for (int vb = 0; vb < C::VBOX_N; ++vb)
-                tma_load_2d(sk + C::OFF_V + vb * C::VBOX + t * 128, &maps.v, vb * 64,
-                            static_cast<int>(r2), &full[st], pol);
+                tma_load_2d(sk + C::OFF_V + vb * C::VBOX + t * 128, &maps.v, vb * 64, rj[s], &full[st], pol);
               if (KI8) {
                 const int m = min(rows_per_box, nj - t);
-                if (m > 0)
-                  bulk_g2s_hint(sk + C::OFF_S + t * 4, sbase + r2 * 4, ((m + 3) & ~3) * 4, &full[st], pol);
+                bulk_g2s_hint(sk + C::OFF_S + t * 4, sbase + static_cast<long long>(rj[s]) * 4, ((m + 3) & ~3) * 4,
+                              &full[st], pol);
               }
             }
             bulk_g2s(sk + C::OFF_QS, qbase + static_cast<long long>(qj) * 2, C::QB, &full[st]);
