@@ -52,6 +52,7 @@ namespace {
 constexpr int kChunk = 64;                  // tokens per unit / pipeline stage
 constexpr int kCW = 4;                      // consumer warps (16 tokens each)
 constexpr int kThreads = (kCW + 2) * 32;    // + one producer warp + one merger warp
+constexpr int kLenMask = 0x7fffffff;        // a context length; the sign bit marks a clamped one
 constexpr int kMaxSub = 4;                  // pages of 16 tokens in one unit
 constexpr int kMaxBatch = 1024;             // prefix arrays live in shared memory
 constexpr int kCtaSmemTarget = 110 * 1024;  // aim for two CTAs per SM
@@ -133,13 +134,27 @@ __device__ __forceinline__ uint32_t swz(uint32_t row, uint32_t byte) {
   return a;
 }
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
-                                            uint64_t* bar, uint64_t policy) {
+// All column blocks of the map's rows from `row` on: block-major in shared memory.
+__device__ __forceinline__ void tma_load_rows(void* dst, const CUtensorMap* map, int row, uint64_t* bar,
+                                              uint64_t policy) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      ".L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar)), "l"(policy)
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      ".L2::cache_hint [%0], [%1, {%2, %3, %2}], [%4], %5;" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(smem_addr(bar)), "l"(policy)
       : "memory");
+}
+
+// a / b and the rest for 0 <= a, 0 < b: 32-bit wherever the values fit, which
+// is a fraction of the 64-bit sequence's time.
+__device__ __forceinline__ void div_rest(long long a, long long b, long long& q, long long& r) {
+  if (((a | b) >> 32) == 0) {
+    const uint32_t x = static_cast<uint32_t>(a), y = static_cast<uint32_t>(b);
+    q = x / y;
+    r = x - static_cast<uint32_t>(q) * y;
+  } else {
+    q = a / b;
+    r = a - q * b;
+  }
 }
 
 // Position of a unit in the (b, g, chunk) order, walked forward one unit at a time.
@@ -154,12 +169,13 @@ struct Walker {
     }
     b = lo;
     while (pre[b + 1] <= u) ++b;  // empty sequences have pre[b] == pre[b+1]
-    nb = static_cast<int>((pre[b + 1] - pre[b]) / Hkv);
-    const long long off = u - pre[b];
-    g = static_cast<int>(off / nb);
-    chunk = static_cast<int>(off % nb);
-    Lb = lens[b];
-    cp = pre[b] + static_cast<long long>(g) * nb;
+    Lb = lens[b] & kLenMask;
+    nb = (Lb + kChunk - 1) / kChunk;
+    long long gg, ch;
+    div_rest(u - pre[b], nb, gg, ch);
+    g = static_cast<int>(gg);
+    chunk = static_cast<int>(ch);
+    cp = u - ch;
   }
   // Advance to the next unit; only called when one exists.
   __device__ void next(const long long* pre, const int* lens, int Hkv) {
@@ -169,8 +185,8 @@ struct Walker {
     if (++g < Hkv) return;
     g = 0;
     do { ++b; } while (pre[b + 1] == pre[b]);
-    nb = static_cast<int>((pre[b + 1] - pre[b]) / Hkv);
-    Lb = lens[b];
+    Lb = lens[b] & kLenMask;
+    nb = (Lb + kChunk - 1) / kChunk;
     cp = pre[b];
   }
 };
@@ -189,49 +205,236 @@ __device__ __forceinline__ int split_ctas(long long T, int grid) {
   return static_cast<int>(min(static_cast<long long>(grid), max(want, 1LL)));
 }
 
-// CTA owning unit u when CTA c owns [floor(c T / N), floor((c+1) T / N)).
-__device__ __forceinline__ int cta_of(long long u, long long T, int N) {
-  return static_cast<int>(((u + 1) * N - 1) / T);
+// The units of CTA c: [begin(c), begin(c + 1)) with begin(c) = floor(c T / N).
+struct Split {
+  long long T, q, r;  // T = q N + r
+  int N;
+  __device__ Split(long long T_, int grid) : T(T_), N(split_ctas(T_, grid)) { div_rest(T, N, q, r); }
+  __device__ long long begin(int c) const { return c * q + static_cast<uint32_t>(c) * static_cast<uint32_t>(r) / N; }
+  // The CTA that owns unit u: an estimate in floats, then exact steps.
+  __device__ int owner(long long u) const {
+    int c = min(N - 1, static_cast<int>(static_cast<float>(u) * (static_cast<float>(N) / static_cast<float>(T))));
+    while (begin(c + 1) <= u) ++c;
+    while (begin(c) > u) --c;
+    return c;
+  }
+};
+
+// How a warp shares the [G][DV] floats of a merge record: lane l holds NC pieces
+// of VEC consecutive floats, piece i at VEC (l + 32 i), all of one head.  The
+// accesses of a warp are contiguous, in shared and in global memory (E = G DV / 32
+// consecutive floats per lane instead: 16-way bank conflicts; 13.3 against 10.7 us in the example of merge_jobs).
+template <int DV, int G>
+struct Piece {
+  static constexpr int E = G * DV / 32, VEC = E < 4 ? E : 4, NC = E / VEC;
+  static_assert(DV % VEC == 0 && NC * VEC == E, "whole pieces");
+  __device__ static int at(int lane, int i) { return VEC * (lane + 32 * i); }
+  __device__ static int head(int lane, int i) { return at(lane, i) / DV; }
+};
+
+template <int VEC, bool kGlobal>
+__device__ __forceinline__ void ld_piece(const float* src, float* x) {
+  if constexpr (VEC == 4) {
+    const float4* q = reinterpret_cast<const float4*>(src);
+    const float4 v = kGlobal ? __ldcg(q) : *q;
+    x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+  } else {
+    static_assert(VEC == 2, "pieces of two or four floats");
+    const float2* q = reinterpret_cast<const float2*>(src);
+    const float2 v = kGlobal ? __ldcg(q) : *q;
+    x[0] = v.x; x[1] = v.y;
+  }
+}
+template <int VEC>
+__device__ __forceinline__ void st_piece(float* dst, const float* x) {
+  if constexpr (VEC == 4) *reinterpret_cast<float4*>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+  else *reinterpret_cast<float2*>(dst) = make_float2(x[0], x[1]);
 }
 
-// Vectorised copies of a lane's E consecutive floats.
-template <int E>
-__device__ __forceinline__ void ld_cg_vec(const float* src, float* dst) {
-  if constexpr (E % 4 == 0) {
+// x * inv to out[o ..], float32 or bf16 (o is a multiple of VEC: aligned vectors).
+template <int VEC>
+__device__ __forceinline__ void write_piece(const DecodeParams& p, long long o, const float* x, float inv) {
+  float y[VEC];
 #pragma unroll
-    for (int i = 0; i < E; i += 4) {
-      const float4 x = __ldcg(reinterpret_cast<const float4*>(src + i));
-      dst[i] = x.x; dst[i + 1] = x.y; dst[i + 2] = x.z; dst[i + 3] = x.w;
-    }
+  for (int e = 0; e < VEC; ++e) y[e] = x[e] * inv;
+  if (p.out_f32) {
+    st_piece<VEC>(reinterpret_cast<float*>(p.out) + o, y);
   } else {
+    uint32_t w[VEC / 2];
 #pragma unroll
-    for (int i = 0; i < E; i += 2) {
-      const float2 x = __ldcg(reinterpret_cast<const float2*>(src + i));
-      dst[i] = x.x; dst[i + 1] = x.y;
+    for (int e = 0; e < VEC / 2; ++e) w[e] = pack_bf16(y[2 * e], y[2 * e + 1]);
+    __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(p.out) + o;
+    if constexpr (VEC == 4) *reinterpret_cast<uint2*>(d) = make_uint2(w[0], w[1]);
+    else *reinterpret_cast<uint32_t*>(d) = w[0];
+  }
+}
+
+// A record [G][DV] o, [G] m, [G] l from the lane's pieces.
+template <int DV, int G>
+__device__ __forceinline__ void st_record(float* rec, int lane, const float* M, const float* L, const float* out) {
+  using P = Piece<DV, G>;
+#pragma unroll
+  for (int i = 0; i < P::NC; ++i) {
+    const int at = P::at(lane, i), hh = P::head(lane, i);
+    st_piece<P::VEC>(rec + at, out + i * P::VEC);
+    if (at % DV == 0) {
+      rec[G * DV + hh] = M[i];
+      rec[G * DV + G + hh] = L[i];
     }
   }
 }
 
-__device__ __forceinline__ void write_out(const DecodeParams& p, long long o, float v) {
-  if (p.out_f32) reinterpret_cast<float*>(p.out)[o] = v;
-  else reinterpret_cast<__nv_bfloat16*>(p.out)[o] = __float2bfloat16_rn(v);
+// N records REC floats apart in shared memory, merged into the lane's pieces.
+// A record without tokens has m = -inf and weight 0; at least one has tokens.
+template <int DV, int G, int REC, int N>
+__device__ __forceinline__ void merge_records(const float* recs, int lane, float* M, float* L, float* out) {
+  using P = Piece<DV, G>;
+#pragma unroll
+  for (int i = 0; i < P::NC; ++i) {
+    const int at = P::at(lane, i), hh = P::head(lane, i);
+    float f[N];
+    M[i] = -INFINITY;
+    L[i] = 0.f;
+#pragma unroll
+    for (int w = 0; w < N; ++w) M[i] = fmaxf(M[i], recs[w * REC + G * DV + hh]);
+#pragma unroll
+    for (int w = 0; w < N; ++w) {
+      f[w] = fast_exp2(recs[w * REC + G * DV + hh] - M[i]);
+      L[i] += recs[w * REC + G * DV + G + hh] * f[w];
+    }
+#pragma unroll
+    for (int e = 0; e < P::VEC; ++e) out[i * P::VEC + e] = 0.f;
+#pragma unroll
+    for (int w = 0; w < N; ++w) {
+      float x[P::VEC];
+      ld_piece<P::VEC, false>(recs + w * REC + at, x);
+#pragma unroll
+      for (int e = 0; e < P::VEC; ++e) out[i * P::VEC + e] += x[e] * f[w];
+    }
+  }
+}
+
+// The pair's output rows.
+template <int DV, int G>
+__device__ __forceinline__ void write_rows(const DecodeParams& p, int b, int g, int lane, const float* L,
+                                           const float* out) {
+  using P = Piece<DV, G>;
+  const long long obase = (static_cast<long long>(b) * p.Hq + g * G) * DV;
+#pragma unroll
+  for (int i = 0; i < P::NC; ++i)
+    write_piece<P::VEC>(p, obase + P::at(lane, i), out + i * P::VEC, 1.f / L[i]);
+}
+
+// A pair whose partials this CTA, the last to arrive, merges with all its warps.
+struct MergeJob {
+  int b, g, c_first, c_last;
+  long long cp;  // the pair's first unit
+};
+constexpr int kMergeWarps = kCW + 1;
+// partials loaded per round by a warp whose lanes hold E floats of each
+template <int E>
+constexpr int kBatch = E >= 32 ? 1 : (E >= 16 ? 4 : 8);
+
+// Partials CTA c_first + i0, c_first + i0 + step, ... of a pair, merged into the
+// lane's pieces.  Each batch of CB partials is one round of loads (m, l and o
+// together), folded in with an online rescale; every partial holds at least one
+// token, so its m is finite.
+template <int DV, int G, int REC>
+__device__ __forceinline__ void merge_partials(const float* part, const Split& sp, const MergeJob& jb, int i0,
+                                               int step, int lane, float* M, float* L, float* out) {
+  using P = Piece<DV, G>;
+  constexpr int CB = kBatch<P::E>;
+#pragma unroll
+  for (int i = 0; i < P::NC; ++i) {
+    M[i] = -INFINITY;
+    L[i] = 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < P::E; ++i) out[i] = 0.f;
+  for (int b0 = jb.c_first + i0; b0 <= jb.c_last; b0 += CB * step) {
+    float oo[CB][P::E], mm[CB][P::NC], ll[CB][P::NC];
+#pragma unroll
+    for (int k = 0; k < CB; ++k) {
+      const int cc = b0 + k * step;
+      const bool have = cc <= jb.c_last;
+      const float* sl = part + (static_cast<long long>(cc) * 2 + (jb.cp <= sp.begin(cc) ? 0 : 1)) * REC;
+#pragma unroll
+      for (int i = 0; i < P::NC; ++i) {
+        const int hh = P::head(lane, i);
+        mm[k][i] = have ? __ldcg(sl + G * DV + hh) : -INFINITY;
+        ll[k][i] = have ? __ldcg(sl + G * DV + G + hh) : 0.f;
+#pragma unroll
+        for (int e = 0; e < P::VEC; ++e) oo[k][i * P::VEC + e] = 0.f;
+        if (have) ld_piece<P::VEC, true>(sl + P::at(lane, i), oo[k] + i * P::VEC);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < P::NC; ++i) {
+      float Mn = M[i];
+#pragma unroll
+      for (int k = 0; k < CB; ++k) Mn = fmaxf(Mn, mm[k][i]);
+      const float a = M[i] == -INFINITY ? 0.f : fast_exp2(M[i] - Mn);
+      L[i] *= a;
+#pragma unroll
+      for (int e = 0; e < P::VEC; ++e) out[i * P::VEC + e] *= a;
+#pragma unroll
+      for (int k = 0; k < CB; ++k) {
+        const float w = fast_exp2(mm[k][i] - Mn);  // 0 where there is none
+        L[i] += ll[k][i] * w;
+#pragma unroll
+        for (int e = 0; e < P::VEC; ++e) out[i * P::VEC + e] += oo[k][i * P::VEC + e] * w;
+      }
+      M[i] = Mn;
+    }
+  }
+}
+
+__device__ __forceinline__ void merge_sync() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kMergeWarps * 32) : "memory");
+}
+
+// The jobs the merger warp left, by the consumer warps (0 .. 3) and the merger
+// warp (4) together, once all of them are done streaming: warp w merges every
+// fifth partial, then the merger warp the five results.  One warp alone needs a
+// round of dependent loads per CB partials (6 us for the 16 partials of a pair
+// at B = 1, 4000 tokens, 8 kv heads: 14.9 -> 10.7 us a step).
+template <int DV, int G, int REC>
+__device__ __forceinline__ void merge_jobs(const DecodeParams& p, const MergeJob* jobs, const int* n_jobs,
+                                           float* recs, const Split& sp, int w, int lane) {
+  using P = Piece<DV, G>;
+  merge_sync();
+  const int n = *n_jobs;
+  for (int i = 0; i < n; ++i) {
+    const MergeJob jb = jobs[i];
+    float M[P::NC], L[P::NC], out[P::E];
+    merge_partials<DV, G, REC>(p.part, sp, jb, w, kMergeWarps, lane, M, L, out);
+    st_record<DV, G>(recs + w * REC, lane, M, L, out);
+    merge_sync();
+    if (w == kCW) {
+      merge_records<DV, G, REC, kMergeWarps>(recs, lane, M, L, out);
+      write_rows<DV, G>(p, jb.b, jb.g, lane, L, out);
+      if (lane == 0) p.counters[jb.b * p.Hkv + jb.g] = 0;  // ready for the next launch
+    }
+    merge_sync();
+  }
 }
 
 // The merger warp: for every segment of the CTA's range, combine the consumer
 // warps' records; write the output of pairs inside the range, or the partial of
-// pairs that straddle CTAs and, on the last arrival, merge all their partials.
-// Lane l owns E = G*DV/32 consecutive elements of the [G][DV] output, all in
-// head (l*E)/DV.
+// pairs that straddle CTAs and, on the last arrival, merge all their partials
+// (or leave them as a job for all warps if they are many; a CTA has at most two
+// such pairs).
 template <int R, int DV, int G, int KF>
 __device__ void merge_segments(const DecodeParams& p, const float* merge, uint64_t* deposit,
                                uint64_t* mfree, const long long* pre, const int* lens,
-                               long long T, int N, int c, long long u_begin, long long u_end,
-                               int lane) {
+                               const Split& sp, int c, long long u_begin, long long u_end,
+                               MergeJob* jobs, int* n_jobs, int lane) {
   using C = Cfg<R, DV, G, KF>;
-  constexpr bool KI8 = KF != 0;  // quantised keys (int8 or int4)
-  constexpr int E = G * DV / 32;
-  constexpr int CB = E >= 32 ? 2 : (E >= 16 ? 4 : 8);  // segments loaded per batch
-  const int e0 = lane * E, hh = e0 / DV;
+  using P = Piece<DV, G>;
+  // up to this many partials are two rounds of loads of this warp, which is
+  // quicker than waiting for the others (5 partials, B = 1, 270 tokens, 8 kv
+  // heads: 8.0 us a step against 9.6 with all warps)
+  constexpr int kAlone = 2 * kBatch<P::E>;
   if (u_begin == u_end) return;
   Walker wk;
   wk.seek(u_begin, pre, lens, p.B, p.Hkv);
@@ -240,42 +443,20 @@ __device__ void merge_segments(const DecodeParams& p, const float* merge, uint64
     const int buf = seg & 1;
     if (!mbar_wait(&deposit[buf], (seg >> 1) & 1, p.err)) return;
     const float* recs = merge + buf * kCW * C::REC;
-    float f[kCW], M = -INFINITY, L = 0.f;
-#pragma unroll
-    for (int w = 0; w < kCW; ++w) M = fmaxf(M, recs[w * C::REC + G * DV + hh]);
-#pragma unroll
-    for (int w = 0; w < kCW; ++w) {
-      f[w] = fast_exp2(recs[w * C::REC + G * DV + hh] - M);  // 0 for a warp without tokens
-      L += recs[w * C::REC + G * DV + G + hh] * f[w];
-    }
-    float acc[E];
-#pragma unroll
-    for (int i = 0; i < E; ++i) {
-      float a = 0.f;
-#pragma unroll
-      for (int w = 0; w < kCW; ++w) a += recs[w * C::REC + e0 + i] * f[w];
-      acc[i] = a;
-    }
+    float M[P::NC], L[P::NC], acc[P::E];
+    merge_records<DV, G, C::REC, kCW>(recs, lane, M, L, acc);  // m = -inf: a warp without tokens
     __syncwarp();
     if (lane == 0) mbar_arrive(&mfree[buf]);  // records read: the consumers may reuse them
 
     const int pair = wk.b * p.Hkv + wk.g;
     const long long cp = wk.cp;
     const long long seg_end = min(u_end, cp + wk.nb);
-    const int c_first = cta_of(cp, T, N), c_last = cta_of(cp + wk.nb - 1, T, N);
-    const long long obase = (static_cast<long long>(wk.b) * p.Hq + wk.g * G) * DV;
+    const int c_first = cp >= u_begin ? c : sp.owner(cp);
+    const int c_last = cp + wk.nb <= u_end ? c : sp.owner(cp + wk.nb - 1);
     if (c_first == c_last) {
-      const float inv = 1.f / L;
-#pragma unroll
-      for (int i = 0; i < E; ++i) write_out(p, obase + e0 + i, acc[i] * inv);
+      write_rows<DV, G>(p, wk.b, wk.g, lane, L, acc);
     } else {
-      float* mine = p.part + (static_cast<long long>(c) * 2 + (cp <= u_begin ? 0 : 1)) * C::REC;
-#pragma unroll
-      for (int i = 0; i < E; ++i) mine[e0 + i] = acc[i];
-      if (e0 % DV == 0) {
-        mine[G * DV + hh] = M;
-        mine[G * DV + G + hh] = L;
-      }
+      st_record<DV, G>(p.part + (static_cast<long long>(c) * 2 + (cp <= u_begin ? 0 : 1)) * C::REC, lane, M, L, acc);
       __syncwarp();
       int last = 0;
       if (lane == 0) {
@@ -289,53 +470,15 @@ __device__ void merge_segments(const DecodeParams& p, const float* merge, uint64
       last = __shfl_sync(0xffffffffu, last, 0);
       __syncwarp();
       if (last) {
-        // merge the partials of CTAs c_first..c_last: each batch of CB partials
-        // is one round of loads (m, l and o together), folded in with an online
-        // rescale; every partial holds at least one token, so its m is finite
-        auto slot = [&](int cc) {
-          const long long sc = T * cc / N;
-          return p.part + (static_cast<long long>(cc) * 2 + (cp <= sc ? 0 : 1)) * C::REC;
-        };
-        float Mt = -INFINITY, Lt = 0.f;
-        float out[E];
-#pragma unroll
-        for (int i = 0; i < E; ++i) out[i] = 0.f;
-        for (int b0 = c_first; b0 <= c_last; b0 += CB) {
-          float oo[CB][E], mm[CB], ll[CB];
-#pragma unroll
-          for (int k = 0; k < CB; ++k) {
-            mm[k] = -INFINITY;
-            ll[k] = 0.f;
-            if (b0 + k <= c_last) {
-              const float* sl = slot(b0 + k);
-              mm[k] = __ldcg(sl + G * DV + hh);
-              ll[k] = __ldcg(sl + G * DV + G + hh);
-              ld_cg_vec<E>(sl + e0, oo[k]);
-            } else {
-#pragma unroll
-              for (int i = 0; i < E; ++i) oo[k][i] = 0.f;
-            }
-          }
-          float Mn = Mt;
-#pragma unroll
-          for (int k = 0; k < CB; ++k) Mn = fmaxf(Mn, mm[k]);
-          const float a = Mt == -INFINITY ? 0.f : fast_exp2(Mt - Mn);
-          Lt *= a;
-#pragma unroll
-          for (int i = 0; i < E; ++i) out[i] *= a;
-#pragma unroll
-          for (int k = 0; k < CB; ++k) {
-            const float wk2 = (b0 + k <= c_last) ? fast_exp2(mm[k] - Mn) : 0.f;
-            Lt += ll[k] * wk2;
-#pragma unroll
-            for (int i = 0; i < E; ++i) out[i] += oo[k][i] * wk2;
-          }
-          Mt = Mn;
+        const MergeJob jb{wk.b, wk.g, c_first, c_last, cp};
+        if (c_last - c_first < kAlone) {
+          merge_partials<DV, G, C::REC>(p.part, sp, jb, 0, 1, lane, M, L, acc);
+          write_rows<DV, G>(p, wk.b, wk.g, lane, L, acc);
+          if (lane == 0) p.counters[pair] = 0;  // ready for the next launch
+        } else if (lane == 0) {
+          jobs[*n_jobs] = jb;
+          ++*n_jobs;
         }
-        const float inv = 1.f / Lt;
-#pragma unroll
-        for (int i = 0; i < E; ++i) write_out(p, obase + e0 + i, out[i] * inv);
-        if (lane == 0) p.counters[pair] = 0;  // ready for the next launch
       }
     }
     u = seg_end;
@@ -373,10 +516,11 @@ __device__ void prefetch_first_chunks(const DecodeParams& p, int lane, int limit
   }
   const long long T = __shfl_sync(0xffffffffu, inc, 31);
   const long long pre = inc - x;
-  const int N = split_ctas(T, gridDim.x);
   const int c = blockIdx.x;
-  if (T == 0 || c >= N) return;  // warp-uniform
-  const long long u_begin = T * c / N, u_end = T * (c + 1) / N;
+  if (T == 0) return;  // warp-uniform
+  const Split sp(T, gridDim.x);
+  if (c >= sp.N) return;
+  const long long u_begin = sp.begin(c), u_end = sp.begin(c + 1);
   const long long u = u_begin + lane;
   int b = 0;
   for (int bb = 0; bb < B; ++bb) {
@@ -387,8 +531,9 @@ __device__ void prefetch_first_chunks(const DecodeParams& p, int lane, int limit
   const long long pb = __shfl_sync(0xffffffffu, pre, b);
   const int nb = (Lb + kChunk - 1) / kChunk;
   if (lane >= nunits || u >= u_end || nb == 0) return;
-  const long long off = u - pb;
-  const int g = static_cast<int>(off / nb), t0 = static_cast<int>(off % nb) * kChunk;
+  long long gg, ch;
+  div_rest(u - pb, nb, gg, ch);
+  const int g = static_cast<int>(gg), t0 = static_cast<int>(ch) * kChunk;
   auto fetch = [&](long long row, int rows) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const unsigned char*>(p.k) + row * RB),
                  "r"(static_cast<uint32_t>(rows * RB))
@@ -436,6 +581,8 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
   uint64_t* mfree = deposit + 2;                                    // [2] records free
   long long* pre = reinterpret_cast<long long*>(smem + C::OFF_PRE);  // [B+1] (in units)
   int* lens = reinterpret_cast<int*>(pre + (p.B + 1));               // [B]
+  MergeJob* jobs = reinterpret_cast<MergeJob*>(smem + C::OFF_BAR + 256);  // [2]
+  int* n_jobs = reinterpret_cast<int*>(jobs + 2);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x;
@@ -450,6 +597,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
       mbar_init(&deposit[b2], kCW);
       mbar_init(&mfree[b2], 1);
     }
+    *n_jobs = 0;
     fence_barrier_init();
   }
   // ---- clamped context lengths and prefix sums of units
@@ -466,7 +614,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     if (p.fuse_append && L >= 0) ++L;  // the appended token is part of the context
     if (L < 0 || L > limit) {
       record_error(p.err, TK_DEVERR_INDEX);
-      L = L < 0 ? 0 : limit;
+      L = (L < 0 ? 0 : limit) | ~kLenMask;
     }
     lens[b] = L;
   }
@@ -475,7 +623,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     long long run = 0;
     for (int base = 0; base < B; base += 32) {
       const int b = base + lane;
-      const long long x = b < B ? static_cast<long long>((lens[b] + kChunk - 1) / kChunk) * Hkv : 0;
+      const long long x = b < B ? static_cast<long long>(((lens[b] & kLenMask) + kChunk - 1) / kChunk) * Hkv : 0;
       long long inc = x;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
@@ -492,21 +640,23 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
   // Partition over N = split_ctas(T, grid) CTAs: every owning CTA gets at
   // least one unit and the CTAs sharing a pair are consecutive; the rest own
   // nothing.
-  const int N = split_ctas(T, gridDim.x);
-  const long long u_begin = c < N ? T * c / N : T, u_end = c < N ? T * (c + 1) / N : T;
+  const Split sp(T, gridDim.x);
+  const long long u_begin = c < sp.N ? sp.begin(c) : T, u_end = c < sp.N ? sp.begin(c + 1) : T;
+  // Boxes of a chunk: 64 rows, or one per page of 16 or 32 tokens.  A box holds
+  // its rows' 128-byte column blocks one after the other.
+  const int rows_per_box = (p.page_size == 0 || p.page_size >= kChunk) ? kChunk : p.page_size;
 
   if (warp == kCW) {
     // ------------------------------------------------------------------ producer
     const uint64_t pol = l2_policy_evict_first();
-    const unsigned char* sbase = reinterpret_cast<const unsigned char*>(p.k_scale);
     const unsigned char* qbase = static_cast<const unsigned char*>(p.q);
     const int ps = p.page_size;
-    const int rows_per_box = (ps == 0 || ps >= kChunk) ? kChunk : ps;
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.k)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.v)) : "memory");
     }
     bool ok = true;
+    int st = 0, use = 0;  // ring stage, and how often it has been used
     for (long long w0 = u_begin; ok && w0 < u_end; w0 += 32) {
       // lane j prepares unit w0 + j: first cache row of the chunk, valid tokens, query offset
       long long app = -1;
@@ -519,12 +669,13 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
         b = wk.b; g = wk.g;
         t0 = wk.chunk * kChunk;
         n = min(kChunk, wk.Lb - t0);
-        qoff = (b * p.Hq + g * G) * R;
+        // the consumers read the queries at a segment's first chunk only
+        qoff = wk.chunk == 0 || u == u_begin ? (b * p.Hq + g * G) * R : -1;
         // Append fused into the decode: the chunk holding a pair's last token gets
         // the step's new token written at position seq_lens[b] (exactly as the
         // append kernel does) just before its TMA loads are issued; no other CTA
         // reads that chunk.  A clamped length (the token does not fit) gets no write.
-        if (p.fuse_append && wk.chunk + 1 == wk.nb && p.seq_lens[b] == wk.Lb - 1) {
+        if (p.fuse_append && wk.chunk + 1 == wk.nb && lens[b] >= 0) {
           const int pos = wk.Lb - 1;
           if (ps == 0) {
             app = (static_cast<long long>(b) * Hkv + g) * p.capacity + pos;
@@ -559,16 +710,18 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
         }
       }
       const int cnt = static_cast<int>(min(32LL, u_end - w0));
+      const uint32_t appends = __ballot_sync(0xffffffffu, app >= 0);
       for (int j = 0; j < cnt; ++j) {
         int rj[kMaxSub];
 #pragma unroll
-        for (int s = 0; s < kMaxSub; ++s) rj[s] = __shfl_sync(0xffffffffu, row[s], j);
+        for (int s = 0; s < kMaxSub; ++s)
+          rj[s] = s == 0 || rows_per_box < kChunk ? __shfl_sync(0xffffffffu, row[s], j) : 0;
         const int nj = __shfl_sync(0xffffffffu, n, j);
         const int qj = __shfl_sync(0xffffffffu, qoff, j);
-        const int bj = __shfl_sync(0xffffffffu, b, j);
-        const int gj = __shfl_sync(0xffffffffu, g, j);
-        const long long aj = __shfl_sync(0xffffffffu, app, j);
-        if (aj >= 0) {
+        if ((appends >> j) & 1u) {
+          const int bj = __shfl_sync(0xffffffffu, b, j);
+          const int gj = __shfl_sync(0xffffffffu, g, j);
+          const long long aj = __shfl_sync(0xffffffffu, app, j);
           // the new row, then a proxy fence: the TMA reads below see it
           const long long src = static_cast<long long>(bj) * Hkv + gj;
           write_kv_row<R, DV, KF>(const_cast<void*>(p.k), const_cast<void*>(p.v),
@@ -579,38 +732,30 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
           __syncwarp();
           asm volatile("fence.proxy.async.global;" ::: "memory");
         }
-        if (lane == 0) {
-          const long long i = w0 + j - u_begin;
-          const int st = static_cast<int>(i % C::NSTAGE);
-          if (i >= C::NSTAGE && !mbar_wait(&empty[st], ((i / C::NSTAGE) - 1) & 1, p.err)) ok = false;
-          if (ok) {
-            unsigned char* sk = smem + st * C::STAGE;
-            const uint32_t sbytes = KI8 ? ((nj + 3) & ~3) * 4 : 0;
-            // rows_per_box = 64 except for pages of 16 or 32 tokens; nj >= 1
-            const int boxes = (nj + rows_per_box - 1) / rows_per_box;
-            mbar_arrive_expect_tx(&full[st], boxes * rows_per_box * ((C::KB + C::VB) / kChunk) + sbytes + C::QB);
-#pragma unroll
-            for (int s = 0; s < kMaxSub; ++s) {
-              if (s >= boxes) break;
-              const int t = s * rows_per_box;
-#pragma unroll
-              for (int kb = 0; kb < C::KBOX_N; ++kb)
-                tma_load_2d(sk + kb * C::KBOX + t * C::KSW, &maps.k, kb * (C::KSW / (KI8 ? 1 : 2)), rj[s], &full[st],
-                            pol);
-#pragma unroll
-              for (int vb = 0; vb < C::VBOX_N; ++vb)
-                tma_load_2d(sk + C::OFF_V + vb * C::VBOX + t * 128, &maps.v, vb * 64, rj[s], &full[st], pol);
-              if (KI8) {
-                const int m = min(rows_per_box, nj - t);
-                bulk_g2s_hint(sk + C::OFF_S + t * 4, sbase + static_cast<long long>(rj[s]) * 4, ((m + 3) & ~3) * 4,
-                              &full[st], pol);
-              }
-            }
-            bulk_g2s(sk + C::OFF_QS, qbase + static_cast<long long>(qj) * 2, C::QB, &full[st]);
-          }
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (use > 0) ok = mbar_wait_warp(&empty[st], (use - 1) & 1, p.err);
         if (!ok) break;
+        unsigned char* sk = smem + st * C::STAGE;
+        if (lane == 0) {
+          const int boxes = (nj + rows_per_box - 1) / rows_per_box;  // nj >= 1
+          mbar_arrive_expect_tx(&full[st],
+                                boxes * rows_per_box * ((C::KB + C::VB) / kChunk) + (KI8 ? ((nj + 3) & ~3) * 4 : 0) +
+                                    (qj >= 0 ? C::QB : 0));
+#pragma unroll
+          for (int s = 0; s < kMaxSub; ++s) {
+            if (s >= boxes) break;
+            const int t = s * rows_per_box;
+            tma_load_rows(sk + t * C::RB, &maps.k, rj[s], &full[st], pol);
+            tma_load_rows(sk + C::OFF_V + t * (2 * DV), &maps.v, rj[s], &full[st], pol);
+            if (KI8)
+              bulk_g2s_hint(sk + C::OFF_S + t * 4, p.k_scale + rj[s], ((min(rows_per_box, nj - t) + 3) & ~3) * 4,
+                            &full[st], pol);
+          }
+          if (qj >= 0) bulk_g2s(sk + C::OFF_QS, qbase + static_cast<long long>(qj) * 2, C::QB, &full[st]);
+        }
+        if (++st == C::NSTAGE) {
+          st = 0;
+          ++use;
+        }
       }
     }
     return;
@@ -620,14 +765,16 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     // ------------------------------------------------------------------ merger
     // Empty contexts: zero rows (CTA b % grid writes sequence b).
     for (int b = c; b < B; b += gridDim.x) {
-      if (lens[b] != 0) continue;
+      if ((lens[b] & kLenMask) != 0) continue;
       for (int e = lane; e < p.Hq * DV; e += 32) {
         const long long o = static_cast<long long>(b) * p.Hq * DV + e;
         if (p.out_f32) reinterpret_cast<float*>(p.out)[o] = 0.f;
         else reinterpret_cast<__nv_bfloat16*>(p.out)[o] = __float2bfloat16_rn(0.f);
       }
     }
-    merge_segments<R, DV, G, KF>(p, merge, deposit, mfree, pre, lens, T, N, c, u_begin, u_end, lane);
+    if (u_begin == u_end) return;
+    merge_segments<R, DV, G, KF>(p, merge, deposit, mfree, pre, lens, sp, c, u_begin, u_end, jobs, n_jobs, lane);
+    merge_jobs<DV, G, C::REC>(p, jobs, n_jobs, merge, sp, kCW, lane);
     return;
   }
 
@@ -644,13 +791,18 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
   bool dead = false;
   Walker wk;
   wk.seek(u_begin, pre, lens, B, Hkv);
+  // this warp's 16 rows: their box, and their place in it
+  const int box = warp * 16 / rows_per_box, in_box = warp * 16 % rows_per_box;
+  const uint32_t k_off = box * rows_per_box * C::RB + in_box * C::KSW;
+  const uint32_t v_off = C::OFF_V + box * rows_per_box * (2 * DV) + in_box * 128;
+  const uint32_t k_blk = rows_per_box * C::KSW, v_blk = rows_per_box * 128;  // column block strides
+  int st = 0;
+  uint32_t ph = 0;
 
   for (long long u = u_begin; u < u_end; ++u) {
-    const long long i = u - u_begin;
-    const int st = static_cast<int>(i % C::NSTAGE);
-    if (!dead && !mbar_wait(&full[st], (i / C::NSTAGE) & 1, p.err)) dead = true;
+    if (!dead && !mbar_wait(&full[st], ph, p.err)) dead = true;
     const unsigned char* sk = smem + st * C::STAGE;
-    const uint32_t k_s = smem_addr(sk), v_s = smem_addr(sk + C::OFF_V);
+    const uint32_t k_s = smem_addr(sk) + k_off, v_s = smem_addr(sk) + v_off;
     const float* ss = reinterpret_cast<const float*>(sk + C::OFF_S);
     const __nv_bfloat16* sq = reinterpret_cast<const __nv_bfloat16*>(sk + C::OFF_QS);
     const bool seg_first = (u == u_begin) || wk.chunk == 0;
@@ -694,12 +846,12 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
       // Ragged chunk: the rows past the context take part in V^T P^T with p = 0,
       // so clear them (unused cache slots may hold non-finite bytes).  A row of a
       // swizzled box is its 128 contiguous bytes, whatever the swizzle.
-      unsigned char* vz = const_cast<unsigned char*>(sk) + C::OFF_V;
+      unsigned char* vz = const_cast<unsigned char*>(sk) + v_off;
       const int nrow = 16 - nvalid;
       for (int e = lane; e < nrow * C::VBOX_N * 8; e += 32) {
-        const int rrow = warp * 16 + nvalid + e / (C::VBOX_N * 8);
+        const int rrow = nvalid + e / (C::VBOX_N * 8);
         const int rest = e % (C::VBOX_N * 8);
-        *reinterpret_cast<uint4*>(vz + (rest / 8) * C::VBOX + rrow * 128 + (rest % 8) * 16) =
+        *reinterpret_cast<uint4*>(vz + (rest / 8) * v_blk + rrow * 128 + (rest % 8) * 16) =
             make_uint4(0u, 0u, 0u, 0u);
       }
       // order these generic-proxy writes before the next TMA write of this stage
@@ -710,13 +862,13 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
       // ---- S^T (16 tokens x 8 heads) = K Q^T
       float s[4] = {0.f, 0.f, 0.f, 0.f};
       const int mi = lane >> 3, rr = lane & 7;
-      const uint32_t krow = warp * 16 + (mi & 1) * 8 + rr;
+      const uint32_t krow = (mi & 1) * 8 + rr;
       if constexpr (!KI8) {
         // bf16 keys: one ldmatrix.x4 per 16-wide k step
 #pragma unroll
         for (int ks = 0; ks < C::KSTEPS; ++ks) {
           const int kc = ks * 2 + (mi >> 1);  // 16-byte chunk of the key row
-          const uint32_t addr = k_s + (kc / (C::KSW / 16)) * C::KBOX +
+          const uint32_t addr = k_s + (kc / (C::KSW / 16)) * k_blk +
                                 swz<C::KSW>(krow, (kc % (C::KSW / 16)) * 16);
           uint32_t a0, a1, a2, a3;
           ldsm_x4(addr, a0, a1, a2, a3);
@@ -738,7 +890,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
 #pragma unroll
           for (int kp = 0; kp < C::KSTEPS / 4; ++kp) {
             const int kc = kp * 2 + (mi >> 1);
-            const uint32_t addr = k_s + (kc / (C::KSW / 16)) * C::KBOX +
+            const uint32_t addr = k_s + (kc / (C::KSW / 16)) * k_blk +
                                   swz<C::KSW>(krow, (kc % (C::KSW / 16)) * 16);
             uint32_t w0, w1, w2, w3;  // (rows 0-7, chunk 2kp), (8-15, 2kp), (0-7, 2kp+1), (8-15, 2kp+1)
             ldsm_x4(addr, w0, w1, w2, w3);
@@ -767,7 +919,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
 #pragma unroll
           for (int kp = 0; kp < C::KSTEPS / 2; ++kp) {
             const int kc = kp * 2 + (mi >> 1);
-            const uint32_t addr = k_s + (kc / (C::KSW / 16)) * C::KBOX +
+            const uint32_t addr = k_s + (kc / (C::KSW / 16)) * k_blk +
                                   swz<C::KSW>(krow, (kc % (C::KSW / 16)) * 16);
             uint32_t w0, w1, w2, w3;  // (rows 0-7, step 2kp), (8-15, 2kp), (0-7, 2kp+1), (8-15, 2kp+1)
             ldsm_x4(addr, w0, w1, w2, w3);
@@ -810,12 +962,12 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
       const uint32_t pb0 = movm_t(pack_bf16(p0, p1));
       const uint32_t pb1 = movm_t(pack_bf16(p2, p3));
       // ---- O^T = alpha O^T + V^T P^T
-      const uint32_t vrow = warp * 16 + (mi >> 1) * 8 + rr;
+      const uint32_t vrow = (mi >> 1) * 8 + rr;
 #pragma unroll
       for (int mt = 0; mt < DV / 16; ++mt) {
         o[mt][0] *= al0; o[mt][1] *= al1; o[mt][2] *= al0; o[mt][3] *= al1;
         const int dc = mt * 2 + (mi & 1);   // 16-byte chunk of the value row (8 values)
-        const uint32_t addr = v_s + (dc / 8) * C::VBOX + swz<128>(vrow, (dc % 8) * 16);
+        const uint32_t addr = v_s + (dc / 8) * v_blk + swz<128>(vrow, (dc % 8) * 16);
         uint32_t a0, a1, a2, a3;
         ldsm_x4_t(addr, a0, a1, a2, a3);
         mma16816(o[mt], a0, a1, a2, a3, pb0, pb1);
@@ -823,6 +975,10 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[st]);
+    if (++st == C::NSTAGE) {
+      st = 0;
+      ph ^= 1u;
+    }
 
     if (seg_last) {
       // ---------------------------------------------------------------- segment end
@@ -865,6 +1021,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     }
     if (u + 1 < u_end) wk.next(pre, lens, Hkv);
   }
+  merge_jobs<DV, G, C::REC>(p, jobs, n_jobs, merge, sp, warp, lane);
 }
 
 // ---------------------------------------------------------------- host side
@@ -882,21 +1039,25 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 2-D map over `rows` rows of `width` elements, box (box_w elements x box_rows rows).
-bool make_map_2d(CUtensorMap* m, const void* base, bool int8, long long width, long long rows,
-                 int box_w, int box_rows, int swizzle_bytes) {
+// Map over `rows` rows of `width` elements as column blocks of block_w elements:
+// dimensions (column in the block, row, block), box (block_w, box_rows, all blocks).
+bool make_row_map(CUtensorMap* m, const void* base, bool int8, long long width, long long rows, int block_w,
+                  int box_rows, int swizzle_bytes) {
   auto enc = encode_fn();
   if (!enc) return false;
   const int es = int8 ? 1 : 2;
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(width), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(width) * es};
-  cuuint32_t box[2] = {static_cast<cuuint32_t>(box_w), static_cast<cuuint32_t>(box_rows)};
-  cuuint32_t estr[2] = {1, 1};
+  const int blocks = static_cast<int>(width / block_w);
+  cuuint64_t dims[3] = {static_cast<cuuint64_t>(block_w), static_cast<cuuint64_t>(rows),
+                        static_cast<cuuint64_t>(blocks)};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(width) * es, static_cast<cuuint64_t>(block_w) * es};
+  cuuint32_t box[3] = {static_cast<cuuint32_t>(block_w), static_cast<cuuint32_t>(box_rows),
+                       static_cast<cuuint32_t>(blocks)};
+  cuuint32_t estr[3] = {1, 1, 1};
   CUtensorMapSwizzle sw = swizzle_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                           : swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                           : swizzle_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B
                                                 : CU_TENSOR_MAP_SWIZZLE_NONE;
-  return enc(m, int8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+  return enc(m, int8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
              const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -912,9 +1073,8 @@ cudaError_t launch_t(const DecodeParams& p, cudaStream_t stream) {
   if (rows >= (1LL << 31)) return cudaErrorInvalidValue;  // TMA row coordinates are 32-bit
   const int box_rows = (p.page_size == 0 || p.page_size >= kChunk) ? kChunk : p.page_size;
   DecodeMaps maps;
-  if (!make_map_2d(&maps.k, p.k, KI8, KF == 2 ? R / 2 : R, rows, C::KSW / (KI8 ? 1 : 2), box_rows,
-                   C::KSW) ||
-      !make_map_2d(&maps.v, p.v, false, DV, rows, 64, box_rows, 128))
+  if (!make_row_map(&maps.k, p.k, KI8, KF == 2 ? R / 2 : R, rows, C::KSW / (KI8 ? 1 : 2), box_rows, C::KSW) ||
+      !make_row_map(&maps.v, p.v, false, DV, rows, 64, box_rows, 128))
     return cudaErrorInvalidValue;
   auto kern = decode_kernel<R, DV, G, KF>;
   const int smem = C::OFF_PRE + (p.B + 1) * 8 + p.B * 4 + 1024;  // + alignment slack
