@@ -15,9 +15,9 @@
 // dimension and the TMEM lanes: thread t of a 4-warp group owns key t.  The
 // CTA visits every 128-query tile i (i >= j when causal) of each of the G
 // query heads of g, as two 64-query halves h:
-//   warp 9 (one lane): TMA loads of K_j, V_j (once) and, per half tile, of
-//       Q, dO and the rows' statistics into a 4-slot ring.
-//   warp 8 (whole warp, one elected lane issues): per tile and half
+//   warp 21 (one lane): TMA loads of K_j, V_j (once) and, per half tile, of
+//       Q, dO and the rows' statistics into a ring.
+//   warps 20 and 22 (whole warp, one elected lane issues): per tile and half
 //       S^T_h  = K Q_h^T     (M=128 keys, N=64 queries, K=r)
 //       dP^T_h = V dO_h^T    (M=128, N=64, K=d_v)
 //       dV    += P^T_h dO_h  (N=d_v, K=64; P^T_h read from TMEM)
@@ -25,27 +25,36 @@
 //     and per tile  dQ_i = dS K  (M=128 queries, N=r, K=128 keys; dS from the
 //     same shared-memory tile read MN-major), completion on mbarriers through
 //     tcgen05.commit.  Where TMEM has room for P^T in columns of its own and
-//     shared memory for two dS tiles (the EARLY schedule), the next tile's
-//     S / dP products of a half are issued as soon as the half's softmax warps
-//     have read S / dP into registers, and a tile's dQ product during the next
-//     tile; otherwise each half's products follow its softmax.
-//   warps 0-3 / 4-7 (half 0 / 1): read S^T_h and dP^T_h from TMEM, form
+//     shared memory for two dS tiles (the EARLY schedule), warp 20 issues the next
+//     tile's S / dP products of a half as soon as the half's softmax warps have
+//     read S / dP into registers, and warp 22 all others as their operands arrive;
+//     otherwise warp 20 issues everything, each half's products after its softmax.
+//   warps 0-15 (warps 8 h .. 8 h + 7: half h, 32 of its queries each group of four):
+//       read their part of S^T_h and dP^T_h from TMEM 16 columns at a time, form
 //       P^T = exp2(S^T scale log2e - lse log2e) (masked) and
 //       dS^T = P^T (dP^T - D) in packed fp32 pairs, write P^T as bf16 into
-//       TMEM and dS^T as bf16 into the swizzled shared-memory tile.  Then each
-//       warpgroup adds half of the previous tile's dQ columns (thread t: query
-//       t) into global dq: staged in shared memory, one TMA tensor reduce-add
-//       (cp.reduce.async.bulk.tensor .add) per warp.  At the end warps 0-3
-//       store dK (times scale) and the first half of dV's columns, warps 4-7
-//       the second half.
-// 10 warps, so that a thread may hold 168 registers.
+//       TMEM and dS^T as bf16 into the swizzled shared-memory tile.  At the end they
+//       store dV.
+//   warps 16-19 (thread: one query): read dQ of each tile from TMEM and add it into
+//       global dq, staged in shared memory, by TMA tensor reduce-adds
+//       (cp.reduce.async.bulk.tensor .add).  At the end they store dK (times scale).
+// What bounds it: the tensor pipe is busy for about 60 % of a tile's time (44 small
+// products, 2000 cycles, those with N = 64 or r limited by reading A from shared
+// memory), the rest are handoffs.  What brought it there (7B shape, B=2, H=32,
+// S=8192, r=32, d_v=128, causal, preprocessing included): dQ read back by warps of
+// its own instead of by the softmax warps (1987 -> 1743 us), sixteen softmax warps
+// with 80 registers instead of eight with 168 and dK / dV through TMA stores
+// (1655), the statistics apart from the tiles and two staging places for dQ (1608).
+// One product of N = 128 for both halves' S^T and dP^T needs fewer reads of K and
+// V, but the halves then run in step and wait together: 1820 us.
 //
 // TMEM columns: [0,64) S^T_0, [64,128) dP^T_0, [128,192) S^T_1,
 // [192,256) dP^T_1, then dV (d_v), dK (r), dQ (r), and where they fit P^T_0,
-// P^T_1 (32 columns each; otherwise P^T_h sits in the first 32 of S^T_h).
+// P^T_1 (32 columns each; otherwise P^T_h sits in S^T_h, each group of four warps'
+// 16 columns over the first half of the 32 it has read itself).
 // At r = 128, dV, dK and dQ do not fit beside the score tiles: dQ_i is then
 // computed over S^T_1 / dP^T_1 once the half-1 softmax has consumed them,
-// warps 4-7 read it back at once, and the next half-1 scores follow.
+// warps 16-19 read it back at once, and the next half-1 scores follow.
 #include <algorithm>
 #include <type_traits>
 
@@ -59,7 +68,12 @@ namespace {
 constexpr int kKeys = 128;         // keys per CTA (MMA M, TMEM lanes)
 constexpr int kQT = 128;           // queries per tile
 constexpr int kHalfQ = 64;         // queries per S / dP half
-constexpr int kTcThreads = 320;    // 2 x 4 softmax warps, the MMA warp, the TMA warp
+// Warps 0-15: softmax gradient, four groups of four: query half 0 / 1, 32 of its
+// 64 queries each; 16-19: dQ; 20: MMA; 21: TMA; 22: the gradients' MMAs where
+// scores are issued early.
+constexpr int kTcThreads = 736;
+constexpr int kTcBound = 768;      // six warps per sub-partition: 80 registers per thread
+constexpr int kWarpDq = 16, kWarpMma = 20, kWarpTma = 21, kWarpMma2 = 22;
 constexpr int kTmemColsTc = 512;
 constexpr int kBoxB = 128 * 128;   // one 64-column (128-byte) box of a 128-row tile
 
@@ -83,35 +97,38 @@ struct TCfg {
   static constexpr int QHB = QK_NBOX * QHBOX;       // Q half tile
   static constexpr int OHB = kHalfQ * DV * 2;       // dO half tile (DV / 64 boxes)
   static constexpr int OBOX = kHalfQ * 128;         // one 64-column box of a dO half tile
-  static constexpr int SL_Q = 0, SL_O = align1k(QHB), SL_L = SL_O + OHB, SL_D = SL_L + kHalfQ * 4;
-  static constexpr int SLOT = align1k(SL_D + kHalfQ * 4);
+  static constexpr int SL_Q = 0, SL_O = align1k(QHB);
+  static constexpr int SLOT = SL_O + OHB;
+  static constexpr int STATS = 2 * kHalfQ * 4;      // a slot's -lse log2 e, then -D, apart from the tiles
   static constexpr int DSB = kKeys * kQT * 2;       // dS^T tile: [2 halves][128 keys][64 queries]
   // dQ of a tile in TMEM: in columns of its own where they fit (r <= 64), else
   // over S^T_1 / dP^T_1 once the half-1 softmax has consumed them (r = 128)
   static constexpr bool DQ_OWN = 256 + DV + 2 * R <= kTmemColsTc;
-  // dQ read back and staged for the TMA reduce-add, boxes of DQ_W fp32
-  // columns x 32 rows (one per warp) swizzled over DQ_SW bytes: with its own
-  // columns each softmax warpgroup takes R / 2 columns after the next tile's
-  // softmax; over S^T_1 / dP^T_1, warps 4-7 take all R at once, right after
-  // their softmax, and stage them 32 columns at a time
-  static constexpr int DQ_W = DQ_OWN ? R / 2 : 32;
+  // dQ read back by the dQ warps and staged for the TMA reduce-add in boxes of
+  // DQ_W fp32 columns x 32 rows (one warp's) swizzled over DQ_SW bytes; where
+  // shared memory holds a whole dQ tile (R <= 64) each box has its own place
+  static constexpr int DQ_W = R < 32 ? R : 32;
   static constexpr int DQ_SW = DQ_W * 4;
-  static constexpr int DQ_LAYOUT_SHIFT = DQ_SW == 128 ? 0 : (DQ_SW == 64 ? 1 : 2);
-  static constexpr int DQB = DQ_OWN ? kQT * R * 4 : 4 * 32 * DQ_SW;
+  static constexpr int DQ_BOX = 32 * DQ_SW;
+  static constexpr int DQ_PLACES = DQ_OWN ? R / DQ_W : 2;   // per warp
+  static constexpr int DQ_LD = DQ_OWN ? DQ_W : 64;          // columns read at a time
+  static constexpr int DQB = 4 * DQ_PLACES * DQ_BOX;
   static constexpr int OFF_K = 0;
   static constexpr int OFF_V = align1k(KB);
   static constexpr int OFF_SL = OFF_V + VB;
   // without the dS tiles: K, V, a ring of n slots, the dQ stage, barriers, alignment slack
-  static constexpr int fixed(int n) { return OFF_SL + n * SLOT + DQB + 256 + 1024; }
+  static constexpr int fixed(int n) { return OFF_SL + n * (SLOT + STATS) + DQB + 256 + 1024; }
   static constexpr int NDS = fixed(4) + 2 * DSB <= 227 * 1024 ? 2 : 1;   // dS^T tiles in flight
   // half-tile slots: 4 (a fifth, where it fits, measured slower), 3 where 4 do not fit
   static constexpr int NSLOT = fixed(4) + NDS * DSB <= 227 * 1024 ? 4 : 3;
   static constexpr int OFF_DS = OFF_SL + NSLOT * SLOT;
   static constexpr int OFF_DQ = OFF_DS + NDS * DSB;
-  static constexpr int OFF_BAR = OFF_DQ + DQB;
+  static constexpr int OFF_ST = OFF_DQ + DQB;
+  static constexpr int OFF_BAR = OFF_ST + NSLOT * STATS;
   // at least 116 KB so that one CTA (and its 512 TMEM columns) sits on an SM alone
   static constexpr int SMEM = std::max(OFF_BAR + 256 + 1024, 116 * 1024);
   static_assert(OFF_BAR + 256 + 1024 <= 227 * 1024, "shared memory");
+  static_assert(OFF_DQ - OFF_SL >= kWarpDq * 4096 + 4 * 8192, "staging places of the epilogue");
   // TMEM columns
   static constexpr int T_S = 0;          // + 128 h: S^T_h
   static constexpr int T_DP = 64;        // + 128 h: dP^T_h
@@ -133,7 +150,7 @@ struct TCfg {
 };
 
 struct TcMaps {
-  CUtensorMap q, k, v, d_out, dq;
+  CUtensorMap q, k, v, d_out, dq, dk, dv;
 };
 
 // TMA tensor reduce-add of a shared-memory box into global memory (bulk group).
@@ -146,33 +163,26 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, const 
 }
 
 
-// 32 consecutive columns at each of two TMEM addresses, one wait.
-__device__ __forceinline__ void tmem_ld32x2(uint32_t ta, uint32_t tb, uint32_t* v) {
+// 16 consecutive columns at each of two TMEM addresses, one wait.
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, uint32_t* v) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
-      "%28, %29, %30, %31}, [%64];\n\t"
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, "
-      "%41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, "
-      "%58, %59, %60, %61, %62, %63}, [%65];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+      "%11, %12, %13, %14, %15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, "
+      "%27, %28, %29, %30, %31}, [%33];\n\t"
       "tcgen05.wait::ld.sync.aligned;"
-      : TK_R8(0), TK_R8(8), TK_R8(16), TK_R8(24), TK_R8(32), TK_R8(40), TK_R8(48), TK_R8(56)
+      : TK_R8(0), TK_R8(8), TK_R8(16), TK_R8(24)
       : "r"(ta), "r"(tb)
       : "memory");
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : TK_R8(0)
-      : "r"(taddr)
-      : "memory");
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), TK_W8(0)
+               : "memory");
 }
-// N consecutive 32-bit columns (N = 8, 16, 32 or 64).
+// N consecutive 32-bit columns (N = 16, 32 or 64).
 template <int N>
 __device__ __forceinline__ void tmem_ld_n(uint32_t taddr, uint32_t* v) {
-  if constexpr (N == 8) tmem_ld8(taddr, v);
-  else if constexpr (N == 16) tmem_ld16(taddr, v);
+  if constexpr (N == 16) tmem_ld16(taddr, v);
   else if constexpr (N == 32) tmem_ld32(taddr, v);
   else tmem_ld64(taddr, v);
 }
@@ -185,26 +195,49 @@ __device__ __forceinline__ float2 f2(uint32_t a, uint32_t b) {
   return make_float2(__uint_as_float(a), __uint_as_float(b));
 }
 
-// N TMEM columns (fp32) of this thread's lane, times `mul`, to dst (16-byte aligned).
-template <int N>
-__device__ __forceinline__ void tmem_rows_out(uint32_t taddr, float* dst, float mul, bool store) {
+// Stages W fp32 columns of a warp's 32 rows (thread: one row) times `mul` as a
+// box of 4 W bytes per row in the matching swizzle, for a TMA store or reduce.
+template <int W>
+__device__ __forceinline__ void stage_rows(unsigned char* box, const uint32_t* w, float mul, int lane) {
+  constexpr int SW = W * 4, SHIFT = SW == 128 ? 0 : 1;
+  static_assert(SW == 128 || SW == 64, "boxes of 32 or 16 columns");
 #pragma unroll
-  for (int c0 = 0; c0 < N; c0 += 32) {
-    constexpr int W = N < 32 ? N : 32;
-    uint32_t v[W];
-    tmem_ld_n<W>(taddr + c0, v);
-    if (store) {
+  for (int c = 0; c < SW / 16; ++c) {
+    const int pc = c ^ ((lane >> SHIFT) & (SW / 16 - 1));
+    *reinterpret_cast<float4*>(box + lane * SW + pc * 16) =
+        make_float4(__uint_as_float(w[4 * c]) * mul, __uint_as_float(w[4 * c + 1]) * mul,
+                    __uint_as_float(w[4 * c + 2]) * mul, __uint_as_float(w[4 * c + 3]) * mul);
+  }
+  fence_proxy_async_smem();
+  __syncwarp();
+}
+
+// N TMEM columns of a warp's 32 rows, times `mul`, to columns x .. x + N of rows
+// row .. row + 31 of a plane by TMA stores of W columns each (rows past the
+// tensor are cut off), staged in two places of 4 KB in turn.  Per-thread row
+// stores instead touch 32 lines each (64 x 32 planes of S = 256: 339 us against 286).
+template <int N, int W>
+__device__ __forceinline__ void store_cols(const CUtensorMap* map, uint32_t taddr, unsigned char* places, float mul,
+                                           int x, int row, int plane, int lane) {
 #pragma unroll
-      for (int c = 0; c < W / 4; ++c)
-        reinterpret_cast<float4*>(dst + c0)[c] =
-            make_float4(__uint_as_float(v[4 * c]) * mul, __uint_as_float(v[4 * c + 1]) * mul,
-                        __uint_as_float(v[4 * c + 2]) * mul, __uint_as_float(v[4 * c + 3]) * mul);
+  for (int c0 = 0; c0 < N; c0 += W) {
+    uint32_t w[W];
+    tmem_ld_n<W>(taddr + c0, w);
+    if (c0 >= 2 * W) {   // the store before last has read this place
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      __syncwarp();
+    }
+    unsigned char* box = places + (c0 / W & 1) * 4096;
+    stage_rows<W>(box, w, mul, lane);
+    if (lane == 0) {
+      tma_store_3d(map, box, x + c0, row, plane);
+      bulk_commit();
     }
   }
 }
 
 template <int R, int DV>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kTcBound, 1)
 bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   using C = TCfg<R, DV>;
   constexpr int NDS = C::NDS;
@@ -250,21 +283,21 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&s_full[s], 1);
-      mbar_init(&p_ready[s], 128);
+      mbar_init(&p_ready[s], 256);
       mbar_init(&p_free[s], 1);
-      mbar_init(&s_free[s], 128);
+      mbar_init(&s_free[s], 256);
     }
     for (int s = 0; s < NDS; ++s) mbar_init(&ds_free[s], 1);
     mbar_init(dq_full, 1);
-    mbar_init(dq_empty, C::DQ_OWN ? 256 : 128);
+    mbar_init(dq_empty, 128);
     mbar_init(acc_full, 1);
     fence_barrier_init();
   }
-  if (warp == 8) {
+  if (warp == kWarpMma) {
     tmem_alloc(tmem_slot, kTmemColsTc);
     tmem_relinquish();
   }
-  if (warp == 9 && lane == 0) {
+  if (warp == kWarpTma && lane == 0) {
     prefetch_map(&maps.q);
     prefetch_map(&maps.k);
     prefetch_map(&maps.v);
@@ -279,7 +312,7 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 9) {
+  if (warp == kWarpTma) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const int kv_plane = b * p.Hkv + g;
@@ -301,8 +334,8 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
         for (int x = 0; x < DV / 64; ++x)
           tma_load_3d(sb + C::SL_O + x * C::OBOX, &maps.d_out, 64 * x, row, bh, &sl_full[sl]);
         const size_t srow = static_cast<size_t>(bh) * p.S_pad + row;
-        bulk_g2s(sb + C::SL_L, p.nl2 + srow, kHalfQ * 4, &sl_full[sl]);
-        bulk_g2s(sb + C::SL_D, p.nd + srow, kHalfQ * 4, &sl_full[sl]);
+        bulk_g2s(smem + C::OFF_ST + sl * C::STATS, p.nl2 + srow, kHalfQ * 4, &sl_full[sl]);
+        bulk_g2s(smem + C::OFF_ST + sl * C::STATS + kHalfQ * 4, p.nd + srow, kHalfQ * 4, &sl_full[sl]);
         issued = u + 1;
       }
       // no copy may still be landing in shared memory when the CTA exits
@@ -311,7 +344,7 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
       for (int u = std::max(0, issued - C::NSLOT); u < issued; ++u)
         mbar_wait(&sl_full[u % C::NSLOT], (u / C::NSLOT) & 1, p.err);
     }
-  } else if (warp == 8) {
+  } else if (warp == kWarpMma || (C::EARLY && warp == kWarpMma2)) {
     // ------------------------------------------------------------------ MMA issuer
     const uint32_t s_base = smem_addr(smem);
     // one descriptor serves a tile read K-major and MN-major: SBO is the stride of
@@ -332,70 +365,70 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
                  k > 0);
       }
 #pragma unroll
-      for (int k = 0; k < DV / 16; ++k)
-        mma_ss_e(tmem + C::T_DP + 128 * h, dV_a.at((k / 4) * kBoxB + (k % 4) * 32),
-                 dO_bk.at(so + (k / 4) * C::OBOX + (k % 4) * 32), C::ID_S, k > 0);
+      for (int k = 0; k < DV / 64; ++k)
+        mma_ss4_e(tmem + C::T_DP + 128 * h, dV_a.at(k * kBoxB), 32, dO_bk.at(so + k * C::OBOX), 32, C::ID_S, k > 0);
       tc_commit_e(&s_full[h]);
     };
     auto issue_dvdk = [&](int t, int h) {  // dV += P^T_h dO_h, dK += dS^T_h Q_h; the slot is then free
       const uint32_t so = slot_of(t, h) * C::SLOT;
       const uint32_t dso = (t % NDS) * C::DSB + h * (C::DSB / 2);
-#pragma unroll
-      for (int kk = 0; kk < kHalfQ / 16; ++kk)
-        mma_ts_e(tmem + C::T_DV, tmem + C::T_P + C::P_STRIDE * h + 8 * kk, dO_bm.at(so + 16 * kk * 128),
-                 C::ID_DV, (t > 0 || h > 0 || kk > 0) ? 1u : 0u);
+      static_assert(kHalfQ == 64, "four K steps per half");
+      const uint32_t acc = (t > 0 || h > 0) ? 1u : 0u;
+      mma_ts4_e(tmem + C::T_DV, tmem + C::T_P + C::P_STRIDE * h, dO_bm.at(so), 16 * 128, C::ID_DV, acc,
+                C::P_OWN ? 16 : 32);
       if (C::P_OWN) tc_commit_e(&p_free[h]);
-#pragma unroll
-      for (int kk = 0; kk < kHalfQ / 16; ++kk)
-        mma_ss_e(tmem + C::T_DK, dS_ak.at(dso + kk * 32), dQ_b.at(so + 16 * kk * C::QK_SW), C::ID_DK,
-                 (t > 0 || h > 0 || kk > 0) ? 1u : 0u);
+      mma_ss4_e(tmem + C::T_DK, dS_ak.at(dso), 32, dQ_b.at(so), 16 * C::QK_SW, C::ID_DK, acc);
       tc_commit_e(&sl_empty[slot_of(t, h)]);
     };
     auto issue_dq = [&](int t) {           // dQ_t = dS K over the 128 keys
       const uint32_t dso = (t % NDS) * C::DSB;
 #pragma unroll
-      for (int k = 0; k < kKeys / 16; ++k)
-        mma_ss_e(tmem + C::T_DQ, dS_am.at(dso + k * 16 * 128), dK_d.at(k * 16 * C::QK_SW), C::ID_DQ, k > 0);
+      for (int k = 0; k < kKeys / 64; ++k)
+        mma_ss4_e(tmem + C::T_DQ, dS_am.at(dso + k * 64 * 128), 16 * 128, dK_d.at(k * 64 * C::QK_SW), 16 * C::QK_SW,
+                  C::ID_DQ, k > 0);
       tc_commit_e(dq_full);
       tc_commit_e(&ds_free[t % NDS]);
     };
     auto wait_all = [&](uint64_t* bar, uint32_t parity) {
-      return __all_sync(0xffffffffu, mbar_wait(bar, parity, p.err));
+      return mbar_wait_warp(bar, parity, p.err);
     };
-    bool ok = wait_all(kv_full, 0) && wait_all(&sl_full[0], 0);
-    if (ok) {
-      tc_fence_after();
-      issue_sdp(0, 0);
-      ok = wait_all(&sl_full[1], 0);
-      tc_fence_after();
-      if (ok) issue_sdp(0, 1);
-    }
-    if constexpr (C::EARLY) {
-      // per tile and half: the next tile's scores as soon as the half's softmax
-      // warps release S / dP, then (half 0) the previous tile's dQ product, then
-      // this tile's dV / dK products when P / dS arrive
-      for (int t = 0; ok && t < n_tiles; ++t) {
-        for (int h = 0; ok && h < 2; ++h) {
-          if (t + 1 < n_tiles) {
-            if (!(ok = wait_all(&s_free[h], t & 1) && wait_all(&sl_full[slot_of(t + 1, h)], slot_par(t + 1, h))))
-              break;
-            tc_fence_after();
-            issue_sdp(t + 1, h);
-          }
-          if (h == 0 && t > 0) {
-            if (t > 1 && !(ok = wait_all(dq_empty, (t - 2) & 1))) break;
-            tc_fence_after();
-            issue_dq(t - 1);
-          }
-          if (!(ok = wait_all(&p_ready[h], t & 1))) break;
-          tc_fence_after();
-          issue_dvdk(t, h);
-        }
-      }
-      if (ok && n_tiles > 1) ok = wait_all(dq_empty, (n_tiles - 2) & 1);
+    bool ok = true;
+    if (warp == kWarpMma) {
+      ok = wait_all(kv_full, 0) && wait_all(&sl_full[0], 0);
       if (ok) {
         tc_fence_after();
-        issue_dq(n_tiles - 1);
+        issue_sdp(0, 0);
+        ok = wait_all(&sl_full[1], 0);
+        tc_fence_after();
+        if (ok) issue_sdp(0, 1);
+      }
+    }
+    if constexpr (C::EARLY) {
+      // Two issuing warps, so that neither waits for what only the other needs.
+      // One: the next tile's scores of each half as soon as its softmax warps
+      // release S / dP.  The other: a tile's dV / dK products when P / dS arrive
+      // (its Q and dO half tiles have landed: its scores were computed), then its
+      // dQ product.
+      if (warp == kWarpMma) {
+        for (int t = 1; ok && t < n_tiles; ++t) {
+          for (int h = 0; ok && h < 2; ++h) {
+            if (!(ok = wait_all(&sl_full[slot_of(t, h)], slot_par(t, h)) && wait_all(&s_free[h], (t - 1) & 1))) break;
+            tc_fence_after();
+            issue_sdp(t, h);
+          }
+        }
+        ok = false;   // the other warp commits the accumulators
+      } else {
+        for (int t = 0; ok && t < n_tiles; ++t) {
+          for (int h = 0; ok && h < 2; ++h) {
+            if (!(ok = wait_all(&p_ready[h], t & 1))) break;
+            tc_fence_after();
+            issue_dvdk(t, h);
+          }
+          if (!ok || (t > 0 && !(ok = wait_all(dq_empty, (t - 1) & 1)))) break;
+          tc_fence_after();
+          issue_dq(t);
+        }
       }
     } else {
       for (int t = 0; ok && t < n_tiles; ++t) {
@@ -425,9 +458,56 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
       }
     }
     if (ok) tc_commit_e(acc_full);
-  } else {
+  } else if (warp >= kWarpDq && warp < kWarpDq + 4) {
+    // ------------------------------------------------------------------ dQ warps
+    // dQ of every tile (thread: query 32 w + lane of the tile, its TMEM lane) read
+    // from TMEM, scaled, staged in shared memory and added into global dq by one
+    // TMA tensor reduce-add per box, so that no warp waits for another.
+    const int w4 = warp & 3;
+    const uint32_t lane_off = static_cast<uint32_t>(w4 * 32) << 16;
+    unsigned char* place = smem + C::OFF_DQ + w4 * (C::DQ_PLACES * C::DQ_BOX);
+    bool pending = false;
+    for (int t = 0; t < n_tiles; ++t) {
+      if (!mbar_wait_warp(dq_full, t & 1, p.err)) break;
+      tc_fence_after();
+      const int row0 = tile_q(t) * kQT + w4 * 32;   // first query of this warp's rows
+#pragma unroll
+      for (int c0 = 0; c0 < R; c0 += C::DQ_LD) {
+        uint32_t w[C::DQ_LD];
+        tmem_ld_n<C::DQ_LD>(tmem + C::T_DQ + c0 + lane_off, w);
+        if (c0 + C::DQ_LD == R) {
+          tc_fence_before();
+          mbar_arrive(dq_empty);
+        }
+        if (row0 >= S) continue;
+        if (c0 % (C::DQ_PLACES * C::DQ_W) == 0) {   // the previous reduce-adds have read their boxes
+          if (lane == 0 && pending) bulk_wait_read_all();
+          __syncwarp();
+        }
+#pragma unroll
+        for (int x = 0; x < C::DQ_LD; x += C::DQ_W) {
+          unsigned char* box = place + (c0 + x) / C::DQ_W % C::DQ_PLACES * C::DQ_BOX;
+          stage_rows<C::DQ_W>(box, w + x, p.scale, lane);
+          if (lane == 0) {
+            tma_reduce_add_3d(&maps.dq, box, c0 + x, row0, b * p.Hq + tile_head(t));
+            bulk_commit();
+            pending = true;
+          }
+        }
+      }
+    }
+    // dK of the CTA's keys (these warps are done before the softmax warps are)
+    const int key0 = j * kKeys + w4 * 32;
+    if (mbar_wait_warp(acc_full, 0, p.err) && key0 < S) {
+      tc_fence_after();
+      store_cols<R, C::DQ_W>(&maps.dk, tmem + C::T_DK + lane_off, smem + C::OFF_SL + kWarpDq * 4096 + w4 * 8192, p.scale, 0, key0,
+                             b * p.Hkv + g, lane);
+    }
+    if (lane == 0) bulk_wait_read_all();
+  } else if (warp < kWarpDq) {
     // ------------------------------------------------------------------ softmax gradient warps
-    const int h = warp >> 2;                      // query half
+    const int h = warp >> 3;                      // query half
+    const int cg = (warp >> 2) & 1;               // which 32 of its queries
     const int kt = (warp & 3) * 32 + lane;        // key of this thread within the tile (TMEM lane)
     const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + C::T_S + 128 * h + lane_off, tD = tmem + C::T_DP + 128 * h + lane_off;
@@ -435,147 +515,68 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     const bool kvalid = j * kKeys + kt < S;
     const float sl2 = p.scale * 1.4426950408889634f;
     const float2 sl2x2 = make_float2(sl2, sl2);
-    bool ok = true, pending = false;
-    // dQ of tile t (thread kt: query kt of the tile), columns [h R/2, (h+1) R/2):
-    // read from TMEM after the next tile's softmax (dq_fetch), then staged in
-    // shared memory and added into global dq by a TMA reduce per warp (its 32
-    // rows), so that no warp waits for another (dq_store).
-    unsigned char* dq_box =
-        smem + C::OFF_DQ + (C::DQ_OWN ? h * (kQT * C::DQ_SW) : 0) + (warp & 3) * (32 * C::DQ_SW);
-    uint32_t wq[C::DQ_W];
-    bool dq_ok = false;
-    auto dq_fetch = [&](int t) {
-      dq_ok = __all_sync(0xffffffffu, ok && mbar_wait(dq_full, t & 1, p.err));
-      if (dq_ok) {
-        tc_fence_after();
-        tmem_ld_n<C::DQ_W>(tmem + C::T_DQ + h * C::DQ_W + lane_off, wq);
-        tc_fence_before();
-        mbar_arrive(dq_empty);
-      }
-    };
-    auto dq_store = [&](int t) {
-      const int row0 = tile_q(t) * kQT + (warp & 3) * 32;   // first query of this warp's rows
-      if (dq_ok && row0 < S) {
-        if (lane == 0 && pending) bulk_wait_read_all();   // the previous reduce has read the box
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < C::DQ_SW / 16; ++c) {
-          const int pc = c ^ ((lane >> C::DQ_LAYOUT_SHIFT) & (C::DQ_SW / 16 - 1));
-          *reinterpret_cast<float4*>(dq_box + lane * C::DQ_SW + pc * 16) =
-              make_float4(__uint_as_float(wq[4 * c]) * p.scale, __uint_as_float(wq[4 * c + 1]) * p.scale,
-                          __uint_as_float(wq[4 * c + 2]) * p.scale, __uint_as_float(wq[4 * c + 3]) * p.scale);
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          tma_reduce_add_3d(&maps.dq, dq_box, h * C::DQ_W, row0, b * p.Hq + tile_head(t));
-          bulk_commit();
-          pending = true;
-        }
-      }
-      if (!dq_ok) ok = false;
-      dq_ok = false;
-    };
-    // r = 128 (dQ over S^T_1 / dP^T_1): warps 4-7 read dQ_t right after their
-    // softmax of tile t, 64 columns at a time (the first half staged before the
-    // second is read), which then releases S^T_1 / dP^T_1 for the next scores;
-    // each half is added into dq DQ_W columns at a time
-    auto dq_all = [&](int t) {
-      static_assert(C::DQ_OWN || R == 128, "dQ over S^T_1 / dP^T_1 is laid out for r = 128");
-      const bool okw = __all_sync(0xffffffffu, ok && mbar_wait(dq_full, t & 1, p.err));
-      const int row0 = tile_q(t) * kQT + (warp & 3) * 32;
-      if (okw) tc_fence_after();
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t w[64];
-        if (okw) {
-          tmem_ld64(tmem + C::T_DQ + 64 * half + lane_off, w);
-          if (half == 1) {
-            tc_fence_before();
-            mbar_arrive(dq_empty);
-          }
-        }
-        if (okw && row0 < S) {
-#pragma unroll
-          for (int ps = 0; ps < 64 / C::DQ_W; ++ps) {
-            if (lane == 0 && pending) bulk_wait_read_all();   // the previous reduce has read the box
-            __syncwarp();
-#pragma unroll
-            for (int c = 0; c < C::DQ_SW / 16; ++c) {
-              const int pc = c ^ ((lane >> C::DQ_LAYOUT_SHIFT) & (C::DQ_SW / 16 - 1));
-              const int e = ps * C::DQ_W + 4 * c;
-              *reinterpret_cast<float4*>(dq_box + lane * C::DQ_SW + pc * 16) =
-                  make_float4(__uint_as_float(w[e]) * p.scale, __uint_as_float(w[e + 1]) * p.scale,
-                              __uint_as_float(w[e + 2]) * p.scale, __uint_as_float(w[e + 3]) * p.scale);
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-              tma_reduce_add_3d(&maps.dq, dq_box, 64 * half + ps * C::DQ_W, row0, b * p.Hq + tile_head(t));
-              bulk_commit();
-              pending = true;
-            }
-          }
-        }
-      }
-      if (!okw) ok = false;
-    };
+    bool ok = true;
     for (int t = 0; t < n_tiles; ++t) {
       const int sl = slot_of(t, h), buf = t % NDS;
       if (ok) {
         ok = mbar_wait(&s_full[h], t & 1, p.err) && mbar_wait(&sl_full[sl], slot_par(t, h), p.err);
-        if (ok && t >= NDS) ok = mbar_wait(&ds_free[buf], ((t / NDS) - 1) & 1, p.err);
+        // (with one dS tile its buffer is asked for as late as possible, below)
+        if (NDS > 1 && ok && t >= NDS) ok = mbar_wait(&ds_free[buf], ((t / NDS) - 1) & 1, p.err);
         ok = __all_sync(0xffffffffu, ok);
       }
       if (ok) {
         tc_fence_after();
-        const unsigned char* sb = smem + C::OFF_SL + sl * C::SLOT;
-        const float* nl2 = reinterpret_cast<const float*>(sb + C::SL_L);
-        const float* nd = reinterpret_cast<const float*>(sb + C::SL_D);
+        const float* nl2 = reinterpret_cast<const float*>(smem + C::OFF_ST + sl * C::STATS);
+        const float* nd = nl2 + kHalfQ;
         unsigned char* ds_row = smem + C::OFF_DS + buf * C::DSB + h * (C::DSB / 2) + kt * 128;
         // keys past S, and keys after the query on the diagonal tile, get weight 0
         const int qlim = (p.causal && tile_q(t) == j) ? kt - h * kHalfQ : 0;  // visible iff column >= qlim
         // warp-uniform choice: both paths issue warp-collective TMEM loads and stores
         const bool masked = __any_sync(0xffffffffu, !kvalid || qlim > 0);
-        auto chunk = [&](auto mask_tag, int c) {
+        auto chunk = [&](auto mask_tag, int c) {   // queries 16 c .. 16 c + 15 of the half
           constexpr bool kMask = decltype(mask_tag)::value;
-          uint32_t v[64];   // [0, 32): S^T, [32, 64): dP^T
-          tmem_ld32x2(tS + 32 * c, tD + 32 * c, v);
-          if (C::EARLY && c == kHalfQ / 32 - 1) {   // S^T_h, dP^T_h may be overwritten
+          uint32_t v[32];   // [0, 16): S^T, [16, 32): dP^T
+          tmem_ld16x2(tS + 16 * c, tD + 16 * c, v);
+          if (C::EARLY && (c & 1)) {   // these columns of S^T_h, dP^T_h may be overwritten
             tc_fence_before();
             mbar_arrive(&s_free[h]);
           }
-          uint32_t pk[16], dk[16];
+          uint32_t pk[8], dk[8];
 #pragma unroll
-          for (int e2 = 0; e2 < 16; ++e2) {
-            const int col = 32 * c + 2 * e2;
+          for (int e2 = 0; e2 < 8; ++e2) {
+            // (pairs: a broadcast 16-byte shared load takes twice the wavefronts per byte)
+            const int col = 16 * c + 2 * e2;
             float2 x = ffma2(f2(v[2 * e2], v[2 * e2 + 1]), sl2x2, *reinterpret_cast<const float2*>(nl2 + col));
             if (kMask) {
               if (!kvalid || col < qlim) x.x = -INFINITY;
               if (!kvalid || col + 1 < qlim) x.y = -INFINITY;
             }
             const float2 pr = make_float2(fast_exp2(x.x), fast_exp2(x.y));
-            const float2 dsv = fmul2(pr, fadd2(f2(v[32 + 2 * e2], v[33 + 2 * e2]),
+            const float2 dsv = fmul2(pr, fadd2(f2(v[16 + 2 * e2], v[17 + 2 * e2]),
                                                *reinterpret_cast<const float2*>(nd + col)));
             pk[e2] = pack2(pr);
             dk[e2] = pack2(dsv);
           }
-          // P^T_h may overwrite the previous tile's only once its dV product has read it
-          if (C::P_OWN && c == 0 && t > 0) {
-            const bool okp = mbar_wait(&p_free[h], (t - 1) & 1, p.err);
+          // P^T_h may overwrite the previous tile's only once its dV product has read
+          // it, dS^T_h its buffer's last tile once its dK and dQ products have
+          if (!(c & 1) && t > 0 && (C::P_OWN || NDS == 1)) {
+            bool okp = true;
+            if (C::P_OWN) okp = mbar_wait(&p_free[h], (t - 1) & 1, p.err);
+            if (NDS == 1) okp = mbar_wait(&ds_free[0], (t - 1) & 1, p.err) && okp;
             if (!__all_sync(0xffffffffu, okp)) ok = false;
           }
-          tmem_st16(tP + 16 * c, pk);
-          // dS^T row kt, queries 32c .. 32c+31 of the half: four 16-byte chunks, SW128 swizzle
+          // over scores that this warp itself has read, where P^T has no columns of its own
+          tmem_st8(tP + (C::P_OWN ? 8 * c : 32 * (c >> 1) + 8 * (c & 1)), pk);
+          // dS^T row kt, queries 16 c .. 16 c + 15 of the half: two 16-byte pieces, SW128 swizzle
 #pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int chunk_i = (4 * c + m) ^ (kt & 7);
+          for (int m = 0; m < 2; ++m) {
+            const int chunk_i = (2 * c + m) ^ (kt & 7);
             *reinterpret_cast<uint4*>(ds_row + chunk_i * 16) =
                 make_uint4(dk[4 * m], dk[4 * m + 1], dk[4 * m + 2], dk[4 * m + 3]);
           }
         };
 #pragma unroll
-        for (int c = 0; c < kHalfQ / 32; ++c) {
+        for (int c = 2 * cg; c < 2 * cg + 2; ++c) {
           if (masked) chunk(std::true_type{}, c);
           else chunk(std::false_type{}, c);
         }
@@ -584,37 +585,21 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
         tc_fence_before();
         mbar_arrive(&p_ready[h]);
       }
-      if constexpr (C::DQ_OWN) {
-        if (t > 0) {
-          dq_fetch(t - 1);
-          dq_store(t - 1);
-        }
-      } else if (h == 1) {
-        dq_all(t);
-      }
     }
-    if (C::DQ_OWN && n_tiles > 0) {
-      dq_fetch(n_tiles - 1);
-      dq_store(n_tiles - 1);
-    }
-    if (pending) bulk_wait_all();
+    // dV of the CTA's keys, 32 columns each group of four warps; the ring and the dS
+    // tiles are free: every product has read them
+    const int key0 = j * kKeys + (warp & 3) * 32, x0 = 32 * (warp >> 2);
     if (ok) ok = mbar_wait(acc_full, 0, p.err);
-    if (__all_sync(0xffffffffu, ok)) {
+    if (__all_sync(0xffffffffu, ok) && key0 < S && x0 < DV) {
       tc_fence_after();
-      const int key = j * kKeys + kt;
-      const size_t kx = (static_cast<size_t>(b) * p.Hkv + g) * S + key;
-      const bool store = key < S;
-      if (h == 0) {
-        tmem_rows_out<R>(tmem + C::T_DK + lane_off, p.dk + kx * R, p.scale, store);
-        tmem_rows_out<DV / 2>(tmem + C::T_DV + lane_off, p.dv + kx * DV, 1.f, store);
-      } else {
-        tmem_rows_out<DV / 2>(tmem + C::T_DV + DV / 2 + lane_off, p.dv + kx * DV + DV / 2, 1.f, store);
-      }
+      store_cols<32, 32>(&maps.dv, tmem + C::T_DV + x0 + lane_off, smem + C::OFF_SL + warp * 4096, 1.f, x0, key0,
+                         b * p.Hkv + g, lane);
     }
+    if (lane == 0) bulk_wait_read_all();
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == kWarpMma) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemColsTc);
   }
@@ -628,7 +613,9 @@ cudaError_t launch_tc(const BackwardParams& p, cudaStream_t stream) {
       !make_map(&maps.k, p.k, R, p.S, p.B * p.Hkv, C::QK_BOXW, kKeys, C::QK_SW) ||
       !make_map(&maps.v, p.v, DV, p.S, p.B * p.Hkv, 64, kKeys, 128) ||
       !make_map(&maps.d_out, p.d_out, DV, p.S, p.B * p.Hq, 64, kHalfQ, 128) ||
-      !make_map(&maps.dq, p.dq, R, p.S, p.B * p.Hq, C::DQ_W, 32, C::DQ_SW, true))
+      !make_map(&maps.dq, p.dq, R, p.S, p.B * p.Hq, C::DQ_W, 32, C::DQ_SW, true) ||
+      !make_map(&maps.dk, p.dk, R, p.S, p.B * p.Hkv, C::DQ_W, 32, C::DQ_SW, true) ||
+      !make_map(&maps.dv, p.dv, DV, p.S, p.B * p.Hkv, 32, 32, 128, true))
     return cudaErrorInvalidValue;
   auto kern = bwd_tc_kernel<R, DV>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);

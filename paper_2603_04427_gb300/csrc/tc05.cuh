@@ -78,11 +78,12 @@ __device__ __forceinline__ void mma_ts_e(uint32_t d, uint32_t a, uint64_t b, uin
       "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Four K steps of D(tmem) (+)= A(tmem) * B(smem desc) with one election: A
-// advances by 8 columns (16 bf16) and B's start address by b_step bytes per
-// step; `accumulate` applies to the first step, the others accumulate.
+// Four K steps of D(tmem) (+)= A(tmem) * B(smem desc) with one election: B's start
+// address advances by b_step bytes per step, A by 8 columns (16 bf16) except that
+// its second pair of steps begins a_gap columns after the first; `accumulate`
+// applies to the first step, the others accumulate.
 __device__ __forceinline__ void mma_ts4_e(uint32_t d, uint32_t a, uint64_t b, uint32_t b_step,
-                                          uint32_t idesc, uint32_t accumulate) {
+                                          uint32_t idesc, uint32_t accumulate, uint32_t a_gap = 16) {
   const uint64_t s = b_step >> 4;
   asm volatile(
       "{\n\t.reg .pred p, t, e;\n\t.reg .b32 l;\n\telect.sync l|e, 0xffffffff;\n\t"
@@ -91,7 +92,22 @@ __device__ __forceinline__ void mma_ts4_e(uint32_t d, uint32_t a, uint64_t b, ui
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %6, %10, t;\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %7, %10, t;\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %8, %10, t;\n\t}" ::"r"(d),
-      "r"(a), "r"(a + 8), "r"(a + 16), "r"(a + 24), "l"(b), "l"(b + s), "l"(b + 2 * s), "l"(b + 3 * s),
+      "r"(a), "r"(a + 8), "r"(a + a_gap), "r"(a + a_gap + 8), "l"(b), "l"(b + s), "l"(b + 2 * s), "l"(b + 3 * s),
+      "r"(accumulate), "r"(idesc)
+      : "memory");
+}
+// The same with A in shared memory: its start address advances by a_step bytes.
+__device__ __forceinline__ void mma_ss4_e(uint32_t d, uint64_t a, uint32_t a_step, uint64_t b, uint32_t b_step,
+                                          uint32_t idesc, uint32_t accumulate) {
+  const uint64_t s = a_step >> 4, u = b_step >> 4;
+  asm volatile(
+      "{\n\t.reg .pred p, t, e;\n\t.reg .b32 l;\n\telect.sync l|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %9, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %10, p;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %10, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %10, t;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %10, t;\n\t}" ::"r"(d),
+      "l"(a), "l"(a + s), "l"(a + 2 * s), "l"(a + 3 * s), "l"(b), "l"(b + u), "l"(b + 2 * u), "l"(b + 3 * u),
       "r"(accumulate), "r"(idesc)
       : "memory");
 }
