@@ -10,20 +10,32 @@ namespace tk {
 // Launch with programmatic stream serialization: the kernel's CTAs may start
 // (and run their prologue up to pdl_wait()) while the previous kernel on the
 // stream finishes.
+// Clusters of `cluster` consecutive CTAs; 1: no clusters.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                       cudaStream_t stream, Args&&... args) {
+cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t stream, int cluster, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (cluster > 1) {
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                       cudaStream_t stream, Args&&... args) {
+  return launch_pdl_cluster(kern, grid, block, smem, stream, 1, static_cast<Args&&>(args)...);
 }
 
 struct DecodeParams {
@@ -92,6 +104,7 @@ struct PrefillParams {
   float scale_log2;
   int num_sms;
   int head_group;  // (b, h) pairs per L2 group, set by the launcher
+  int split;       // CTAs (of one cluster) per query tile pair, set by the launcher
   // cached mode (a chunk of S queries after seq_lens[b] cached tokens):
   // query i of sequence b sits at position seq_lens[b] + i and the keys are
   // the cache's first seq_lens[b] + S tokens (bottom-right causal)

@@ -177,6 +177,119 @@ __device__ __forceinline__ void split_bf16(float2 x, uint32_t& hi, uint32_t& lo)
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
+// ---------------------------------------------------------------- clusters
+constexpr int kMaxSplit = 8;  // CTAs of a cluster
+
+// Barrier of all threads of the cluster; shared-memory writes before it are
+// visible to reads after it in every CTA.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile(
+      "barrier.cluster.arrive.release.aligned;\n\t"
+      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of this CTA's shared-memory address in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float x;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr) : "memory");
+  return x;
+}
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
+  float4 x;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+               : "r"(addr)
+               : "memory");
+  return x;
+}
+
+// Where the CTAs of a split pair leave their partial results, from the start of
+// shared memory: O of both tiles in fp32 ([row][d_v], the 16-byte pieces of a row
+// swizzled by the row), then max and sum per row, then weights of merge_split.
+template <int DV>
+struct Partial {
+  static constexpr int STAT = 2 * kBM * DV * 4;                     // [tile][max, sum][row]
+  static constexpr int WEIGHT = STAT + 4 * kBM * 4;                 // [row][CTA]
+  static constexpr int BYTES = WEIGHT + 2 * kBM * 4;
+  __device__ static int piece(int x, int i, int c) { return ((x * kBM + i) * DV + ((c ^ (i & 7)) << 2)) * 4; }
+};
+
+// This CTA's share of the pair's rows (rank, rank + C, ... of those in the
+// sequence) merged from the C CTAs' partials and written out, by the 256 softmax
+// threads: first the weights 2^(max - largest) / sum of every row, then 16-byte
+// pieces, 16 loads in flight a thread (row by row, with each row's loads waiting
+// for its weights, a merge of 256 rows took 8 us).
+template <int DV, int C>
+__device__ __forceinline__ void merge_split(const PrefillParams& p, unsigned char* smem, int rank, int qa, int bh,
+                                            int tid) {
+  using P = Partial<DV>;
+  constexpr int PIECES = DV / 4, U = 16 / C;
+  const int rows = (min(2 * kBM, p.S - qa * kBM) - rank + C - 1) / C;  // of this CTA
+  const uint32_t base = smem_addr(smem);
+  float* weight = reinterpret_cast<float*>(smem + P::WEIGHT);
+  if (tid < rows) {
+    const int rr = rank + tid * C, x = rr / kBM, i = rr % kBM;
+    const uint32_t st = base + P::STAT + (x * 2 * kBM + i) * 4;
+    float m[C], l[C], mx = -INFINITY, sum = 0.f;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      m[c] = ld_cluster_f32(cluster_addr(st, c));
+      l[c] = ld_cluster_f32(cluster_addr(st + kBM * 4, c));
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) mx = fmaxf(mx, m[c]);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      m[c] = m[c] == -INFINITY ? 0.f : fast_exp2(m[c] - mx);  // -inf: no key of the row there
+      if (m[c] != 0.f) sum += l[c] * m[c];
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c) weight[tid * C + c] = m[c] / sum;
+  }
+  asm volatile("bar.sync 1, 256;" ::: "memory");
+  for (int q0 = tid; q0 < rows * PIECES; q0 += 256 * U) {
+    float4 y[U][C];
+    float w[U][C];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = min((q0 + 256 * u) / PIECES, rows - 1), rr = rank + k * C;
+      const uint32_t at = base + P::piece(rr / kBM, rr % kBM, tid % PIECES);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        w[u][c] = weight[k * C + c];
+        y[u][c] = ld_cluster_f32x4(cluster_addr(at, c));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = (q0 + 256 * u) / PIECES;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        if (w[u][c] != 0.f) {  // what a CTA without keys of the row holds may be anything
+          o.x += w[u][c] * y[u][c].x;
+          o.y += w[u][c] * y[u][c].y;
+          o.z += w[u][c] * y[u][c].z;
+          o.w += w[u][c] * y[u][c].w;
+        }
+      }
+      if (k >= rows) continue;
+      const size_t e = (static_cast<size_t>(bh) * p.S + qa * kBM + rank + k * C) * DV + 4 * (tid % PIECES);
+      if (p.out_f32) {
+        *reinterpret_cast<float4*>(static_cast<float*>(p.out) + e) = o;
+      } else {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(o.x, o.y), b = __floats2bfloat162_rn(o.z, o.w);
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.out) + e) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      }
+    }
+  }
+}
+
 struct Maps {
   CUtensorMap q, k, v;
   CUtensorMap klo;  // lo plane of widened quantised keys (two K tiles per stage)
@@ -194,7 +307,11 @@ struct Maps {
 //   warps 4-7: the same for tile B
 //   warp 8: TMA producer (Q tiles once, K/V tiles into an NST-stage ring)
 //   warp 9: MMA issuer
-template <int R, int DV, int KF>
+// SPLIT: the CTAs of a cluster compute the same two query tiles, each over its
+// share of the kv tiles, and merge their partial results through distributed
+// shared memory at the end; for launches of so few query tiles that SMs would stay
+// idle (choose_split).
+template <int R, int DV, int KF, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   using C = PCfg<R, DV, KF>;
@@ -221,8 +338,10 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   const int BH = p.B * p.Hq;
   // CTA order: heads in groups of p.head_group whose K/V stay in L2 together;
   // inside a group the heaviest (latest) tile pairs first.
-  const int grp = static_cast<int>(blockIdx.x / (p.head_group * n_tp));
-  const int rem = static_cast<int>(blockIdx.x - static_cast<long>(grp) * p.head_group * n_tp);
+  const uint32_t work = SPLIT ? blockIdx.x / p.split : blockIdx.x;
+  const int rank = SPLIT ? static_cast<int>(blockIdx.x % p.split) : 0;   // = the rank in the cluster
+  const int grp = static_cast<int>(work / (p.head_group * n_tp));
+  const int rem = static_cast<int>(work - static_cast<long>(grp) * p.head_group * n_tp);
   const int gsize = min(p.head_group, BH - grp * p.head_group);
   const int tp = n_tp - 1 - rem / gsize;
   const int bh = grp * p.head_group + rem % gsize;
@@ -274,9 +393,17 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     const int last = L0 + min(qt * kBM + kBM, p.S) - 1;
     return p.causal ? min(n_kv_all, last / kBN + 1) : n_kv_all;
   };
-  const int n_a = tiles_for(qa);
-  const int n_b = has_b ? tiles_for(qb) : 0;
-  const int n_kv = max(n_a, n_b);
+  int n_a = tiles_for(qa);
+  int n_b = has_b ? tiles_for(qb) : 0;
+  int n_kv = max(n_a, n_b);
+  int j0 = 0;  // this CTA's kv tiles: j0 .. j0 + n_kv - 1, counted from j0 below
+  if constexpr (SPLIT) {
+    j0 = n_kv * rank / p.split;
+    const int j1 = n_kv * (rank + 1) / p.split;
+    n_a = max(0, min(n_a, j1) - j0);
+    n_b = max(0, min(n_b, j1) - j0);
+    n_kv = j1 - j0;
+  }
 
   __syncthreads();
   // after the barrier, so that every CTA of this grid holds its TMEM before a
@@ -290,13 +417,13 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   // hold anything there, and 0 * NaN would spread) and then publishes it on
   // k_full.  Other tiles go straight from the TMA to k_full.
   const bool relay = p.seq_lens != nullptr;
-  auto relayed = [&](int j) { return relay && kv_len - j * kBN < kBN; };
+  auto relayed = [&](int j) { return relay && kv_len - (j0 + j) * kBN < kBN; };
   auto finish = [&](int j) -> bool {
     const int st = j % NST;
     unsigned char* sv = smem + C::OFF_K + st * C::STAGE + C::VOFF;
     const bool okc = mbar_wait(&c_full[st], 0, p.err) && mbar_wait(&v_full[st], (j / NST) & 1, p.err);
     if (!__all_sync(0xffffffffu, okc)) return false;
-    const int first = max(kv_len - j * kBN, 0);
+    const int first = max(kv_len - (j0 + j) * kBN, 0);
     const int per_box = (kBN - first) * 8;   // 16-byte pieces per value box
     for (int c = lane; c < per_box * C::V_NBOX; c += 32) {
       const int box = c / per_box, rem2 = c % per_box;
@@ -317,7 +444,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     const int g = h / (p.Hq / p.Hkv);
     const int bps = (p.page_size == 0 || p.page_size >= kBN) ? kBN : p.page_size;
     const int nsub = kBN / bps;
-    if (lane == 0) {
+    if (lane == 0 && n_kv > 0) {
       mbar_arrive_expect_tx(q_full, has_b ? 2 * C::QB : C::QB);
       for (int x = 0; x < (has_b ? 2 : 1); ++x)
         for (int i = 0; i < C::QK_NBOX; ++i)
@@ -330,9 +457,10 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       const int st = j % NST;
       const uint32_t pe = ((j / NST) - 1) & 1;
       // lane s < nsub finds the plane and first row of sub-box s
-      int plane = kv_plane, row = j * kBN;
+      const int tok = (j0 + j) * kBN;  // first key of the tile
+      int plane = kv_plane, row = tok;
       if (p.page_size != 0) {
-        const int t = j * kBN + lane * bps;
+        const int t = tok + lane * bps;
         int page = -1;  // keys past the sequence's pages read the zero fill
         if (lane < nsub && t < kv_len) {
           page = p.page_table[static_cast<long long>(b) * p.max_pages + (t >> p.page_shift)];
@@ -359,9 +487,9 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       } else if (lane == 0) {
         // widened keys from the workspace: [B*Hkv][kw_rows][r] planes, one box per tile
         for (int i = 0; i < C::QK_NBOX; ++i) {
-          tma_load_3d(sk + i * C::QK_BOXB, &maps.k, i * C::QK_BOX, j * kBN, kv_plane, kb);
+          tma_load_3d(sk + i * C::QK_BOXB, &maps.k, i * C::QK_BOX, tok, kv_plane, kb);
           if constexpr (C::KT == 2)
-            tma_load_3d(sk + C::KBA + i * C::QK_BOXB, &maps.klo, i * C::QK_BOX, j * kBN, kv_plane, kb);
+            tma_load_3d(sk + C::KBA + i * C::QK_BOXB, &maps.klo, i * C::QK_BOX, tok, kv_plane, kb);
         }
       }
       if (j >= NST && !mbar_wait_warp(&v_empty[st], pe, p.err)) return false;
@@ -369,10 +497,10 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
         if constexpr (C::SCALE_IN_SOFTMAX) {
           // the tile's key scales (rows past kw_rows are never weighted); their buffer
           // is free with V's: the softmax has read them before it publishes P
-          const uint32_t bytes = static_cast<uint32_t>(min(kBN, p.kw_rows - j * kBN)) * 4u;
+          const uint32_t bytes = static_cast<uint32_t>(min(kBN, p.kw_rows - tok)) * 4u;
           mbar_arrive_expect_tx(&sc_full[st], bytes);
           bulk_g2s(smem + C::OFF_SC + st * C::SCB,
-                   p.kw_scale + static_cast<size_t>(kv_plane) * p.kw_rows + j * kBN, bytes, &sc_full[st]);
+                   p.kw_scale + static_cast<size_t>(kv_plane) * p.kw_rows + tok, bytes, &sc_full[st]);
         }
         mbar_arrive_expect_tx(&v_full[st], C::VB);
       }
@@ -417,11 +545,11 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
         mma_ts4_e(tmem + 256 + x * 128, tmem + x * 128 + 32 * part, dv.at(st * C::STAGE + part * (64 * 128)),
                   16 * 128, C::IDESC_O, (first && part == 0) ? 0u : 1u);
       };
-      bool ok = mbar_wait_warp(q_full, 0, p.err) && mbar_wait_warp(&k_full[0], 0, p.err);
+      bool ok = n_kv > 0 && mbar_wait_warp(q_full, 0, p.err) && mbar_wait_warp(&k_full[0], 0, p.err);
       if (ok) {
         tc_fence_after();
-        issue_s(0, 0);
-        if (has_b) issue_s(1, 0);
+        if (n_a > 0) issue_s(0, 0);
+        if (n_b > 0) issue_s(1, 0);
         tc_commit_e(&k_empty[0]);
       }
       for (int j = 0; ok && j < n_kv; ++j) {
@@ -472,7 +600,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       ok = mbar_wait(&s_full[x], j & 1, p.err);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after();
-      const int kv0 = j * kBN;
+      const int kv0 = (j0 + j) * kBN;
       const bool masked = (p.causal && kv0 + kBN - 1 > L0 + qt * kBM) || (kv0 + kBN > kv_len);
       const int lim = min(kv_len - kv0, p.causal ? pos - kv0 + 1 : kBN);  // visible columns
       // the whole S row of this thread: 128 fp32 scores
@@ -517,7 +645,9 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       l *= alpha;
       // P = exp2(s * scale log2e - m) as bf16 pairs into TMEM columns [0, 64) of S,
       // published in kParts consecutive key ranges
-      const float2 sl2x2 = make_float2(sl2, sl2), negm2 = make_float2(-m_used, -m_used);
+      // (a CTA of a split pair may see no key of a row so far: max -inf, weights 0)
+      const float neg = SPLIT && m_used == -INFINITY ? 0.f : -m_used;
+      const float2 sl2x2 = make_float2(sl2, sl2), negm2 = make_float2(neg, neg);
       float2 acc[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                        make_float2(0.f, 0.f)};
       static_assert(kParts == 2, "two key ranges of P");
@@ -564,6 +694,32 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       const float2 s01 = fadd2(acc[0], acc[1]), s23 = fadd2(acc[2], acc[3]);
       l += (s01.x + s01.y) + (s23.x + s23.y);
     }
+    if constexpr (SPLIT) {
+      // Partial result of this CTA (Partial) over the ring and the Q tiles, once both
+      // tiles' products and so all loads are complete; max -inf where this CTA had no
+      // kv tile for the row.
+      static_assert(Partial<DV>::BYTES <= C::OFF_SC, "partials over the ring and the Q tiles");
+      if (ok || nx == 0) {
+        ok = (n_a == 0 || mbar_wait(&o_full[0], 0, p.err)) && (n_b == 0 || mbar_wait(&o_full[1], 0, p.err));
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      float* stat = reinterpret_cast<float*>(smem + Partial<DV>::STAT) + x * 2 * kBM;
+      const int i = tid & 127;
+      stat[i] = ok && nx > 0 ? m_used : -INFINITY;
+      stat[kBM + i] = l;
+      if (ok && nx > 0 && qt * kBM + (warp & 3) * 32 < p.S) {
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < DV; c0 += 32) {
+          uint32_t o[32];
+          tmem_ld32(tO + lane_off + c0, o);
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            *reinterpret_cast<uint4*>(smem + Partial<DV>::piece(x, i, c0 / 4 + c)) =
+                make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+        }
+      }
+    } else {
     // epilogue: out = O / l
     if (ok) ok = mbar_wait(&o_full[x], 0, p.err);
     if (__all_sync(0xffffffffu, ok)) {
@@ -623,6 +779,16 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       }
       if (lane == 0) bulk_wait_read_all();
     }
+    }
+  }
+  if constexpr (SPLIT) {
+    cluster_sync();
+    if (warp < 8) {
+      if (p.split == 2) merge_split<DV, 2>(p, smem, rank, qa, bh, tid);
+      else if (p.split == 4) merge_split<DV, 4>(p, smem, rank, qa, bh, tid);
+      else merge_split<DV, 8>(p, smem, rank, qa, bh, tid);
+    }
+    cluster_sync();  // no CTA leaves while others read its shared memory
   }
   tc_fence_before();
   __syncthreads();
@@ -706,6 +872,21 @@ __global__ void __launch_bounds__(256) key_widen_kernel(const PrefillParams p, _
 
 // ---------------------------------------------------------------- host side
 
+// CTAs per query tile pair: as many as find an SM each, where the kv tiles saved
+// (about 1 us each) are worth the merge (3 to 4 us), and every CTA keeps three.
+// Not where the row logsumexp is wanted: a training step's forward keeps one order
+// of sums whatever its batch.  Measured, r = 32, d_v = 128, one CTA a pair against
+// split: 32/8 heads, 500 tokens after 8000 82 us -> 51 (two CTAs), 23 after 13000
+// 100 -> 35 (four); 16/8 heads, B=2, 500 after 2000, int8 35 -> 30; but 500 after 500
+// (8 kv tiles) 16.8 -> 18.0 and a prompt of 512 (4) 9.6 -> 12.0.
+int choose_split(const PrefillParams& p, long pairs) {
+  const long kv_tiles = ((p.seq_lens ? p.kv_limit : p.S) + kBN - 1) / kBN;
+  if (p.lse || kv_tiles < 10) return 1;
+  int split = 1;
+  while (2 * split <= kMaxSplit && pairs * 2 * split <= p.num_sms && kv_tiles >= 6 * split) split *= 2;
+  return split;
+}
+
 template <int R, int DV, int KF>
 cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   using C = PCfg<R, DV, KF>;
@@ -743,13 +924,14 @@ cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
       ok = ok && make_map(&maps.klo, lo, R, p.kw_rows, p.B * p.Hkv, C::QK_BOX, kBN, C::QK_SW);
   }
   if (!ok) return cudaErrorInvalidValue;
-  auto kern = prefill_kernel<R, DV, KF>;
-  const int smem = C::SMEM;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
   const long n_qt = (p.S + kBM - 1) / kBM;
   const long grid = (n_qt + 1) / 2 * p.B * p.Hq;  // one CTA per query tile pair
   if (grid > 0x7fffffffL) return cudaErrorInvalidConfiguration;
+  pp.split = choose_split(p, grid);
+  auto kern = pp.split > 1 ? prefill_kernel<R, DV, KF, true> : prefill_kernel<R, DV, KF, false>;
+  const int smem = C::SMEM;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
   if constexpr (KF != kKeyBF16) {
     const long long n = static_cast<long long>(p.B) * p.Hkv * p.kw_rows * (R / 8);
     e = launch_pdl(key_widen_kernel<R, KF, C::KT>, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, stream,
@@ -759,7 +941,8 @@ cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   // about 48 MB of K/V per head group
   const long head_bytes = static_cast<long>(p.seq_lens ? p.kv_limit : p.S) * (R + DV) * 2;
   pp.head_group = static_cast<int>(std::max(1L, std::min<long>(p.B * p.Hq, (48L << 20) / head_bytes)));
-  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(kThreads), smem, stream, maps, pp);
+  return launch_pdl_cluster(kern, dim3(static_cast<unsigned>(grid * pp.split)), dim3(kThreads), smem, stream, pp.split,
+                            maps, pp);
 }
 
 template <int R, int DV>

@@ -1,0 +1,93 @@
+"""Prefill of few query tiles: the kv tiles of a pair split over a cluster.
+
+Launches with at most half as many query tile pairs as SMs, and at least ten kv
+tiles, split a pair's kv tiles over 2, 4 or 8 CTAs, which merge through
+distributed shared memory.  Covered:
+every split, shares without a tile for query tile A or for any (causal pairs
+early in the sequence), rows that a share sees nothing of (contexts that end
+off a tile boundary), every output type, key format, r / d_v staging layout,
+and that a sequence's result does not depend on the split beyond rounding.
+"""
+
+import math
+
+import pytest
+import torch
+
+from _helpers import f64, parity, parity_bf16, require_gpu
+from oracle import attention as oa
+from oracle import cache as oc
+from paper_2603_04427_gb300 import binding as tb
+from paper_2603_04427_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,hq,hkv,S,r,dv,bf16,causal", [
+    (1, 4, 4, 1281, 32, 128, False, True),    # 24 pairs, 11 kv tiles: split 2
+    (1, 2, 1, 1700, 16, 64, True, True),      # 14 kv tiles: split 4
+    (1, 1, 1, 3100, 64, 128, False, True),    # 25 kv tiles: split 8
+    (1, 1, 1, 4097, 32, 128, True, True),     # 33 kv tiles: split 8
+    (1, 2, 2, 1300, 128, 128, False, False),  # full attention
+    (1, 1, 1, 1921, 128, 64, False, False),   # a last pair of one row
+])
+def test_prefill_split(B, hq, hkv, S, r, dv, bf16, causal):
+    require_gpu()
+    q = inputs.normal_bf16((B, hq, S, r), 91, device="cuda")
+    k = inputs.normal_bf16((B, hkv, S, r), 92, device="cuda")
+    v = inputs.normal_bf16((B, hkv, S, dv), 93, device="cuda")
+    out = torch.full((B, hq, S, dv), float("nan"), device="cuda", dtype=torch.bfloat16 if bf16 else torch.float32)
+    tb.tk_attn_prefill(q, k, v, out, causal=causal)
+    assert tb.tk_get_device_error() == 0
+    ref = oa.attention_prefill(f64(q), f64(k), f64(v), 1 / math.sqrt(r), causal=causal)
+    (parity_bf16 if bf16 else parity)(f64(out), ref, what=f"split prefill S={S} r={r} d_v={dv}")
+
+
+@pytest.mark.parametrize("hq,hkv,S,lens,r,dv,page,keys", [
+    (4, 2, 23, [3001, 1], 32, 128, 0, "bf16"),     # one query tile, split 8 and mostly empty shares
+    (4, 1, 130, [2000, 777], 64, 64, 16, "bf16"),  # two tiles, the second of two rows
+    (2, 2, 300, [1111], 32, 128, 64, "int8"),      # hi + lo keys
+    (2, 1, 200, [1500], 128, 128, 0, "int4"),      # scales in the softmax
+    (8, 2, 256, [130, 1200], 16, 128, 128, "bf16"),
+])
+def test_chunk_split(hq, hkv, S, lens, r, dv, page, keys):
+    require_gpu()
+    B, L = len(lens), max(lens) + S
+    cap = (L + 15) // 16 * 16
+    kw = dict(k_int8=keys == "int8", k_int4=keys == "int4")
+    if page:
+        table, n = inputs.paged_layout([x + S for x in lens], page, seed=95)
+        cache = tb.ThinKeyCache.allocate(B, hq, hkv, r, dv, page_size=page, num_pages=n, page_table=table, **kw)
+    else:
+        cache = tb.ThinKeyCache.allocate(B, hq, hkv, r, dv, capacity=cap, **kw)
+    k = inputs.normal_bf16((B, hkv, L, r), 96, device="cuda")
+    v = inputs.normal_bf16((B, hkv, L, dv), 97, device="cuda")
+    q = inputs.normal_bf16((B, hq, S, r), 98, device="cuda")
+    zero = torch.zeros(B, dtype=torch.int32, device="cuda")
+    sl = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    kn = torch.stack([k[b, :, n:n + S] for b, n in enumerate(lens)])
+    vn = torch.stack([v[b, :, n:n + S] for b, n in enumerate(lens)])
+    if not page:
+        tb.tk_kv_append(cache, k[:, :, :max(lens)].contiguous(), v[:, :, :max(lens)].contiguous(), zero)
+    else:   # sequence by sequence: only its own tokens have pages
+        for b, n in enumerate(lens):
+            one = tb.ThinKeyCache(type(cache.desc).from_buffer_copy(cache.desc), cache.k, cache.v, cache.k_scale,
+                                  cache.page_table[b:b + 1].contiguous())
+            one.desc.batch = 1
+            tb.tk_kv_append(one, k[b:b + 1, :, :n].contiguous(), v[b:b + 1, :, :n].contiguous(), zero[:1])
+    out = torch.full((B, hq, S, dv), float("nan"), device="cuda")
+    tb.tk_attn_prefill_cached(cache, q, kn, vn, sl, L, out)
+    assert tb.tk_get_device_error() == 0
+    kq = f64(k)
+    if keys == "int8":
+        code, scale = oc.quantize_int8_per_token(kq)
+        kq = code * scale[..., None].astype(float)
+    elif keys == "int4":
+        code, scale = oc.quantize_int4_per_token(kq)
+        kq = code * scale[..., None].astype(float)
+    G = hq // hkv
+    for b, n in enumerate(lens):
+        for h in range(hq):
+            ref = oa.attention_head(f64(q[b, h]), kq[b, h // G, :n + S], f64(v[b, h // G, :n + S]),
+                                    1 / math.sqrt(r), causal_offset=n)
+            parity(f64(out[b, h]), ref, what=f"split chunk b={b} h={h} {keys} r={r} page={page}")
