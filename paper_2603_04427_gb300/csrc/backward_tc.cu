@@ -56,6 +56,7 @@
 // computed over S^T_1 / dP^T_1 once the half-1 softmax has consumed them,
 // warps 16-19 read it back at once, and the next half-1 scores follow.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -236,7 +237,74 @@ __device__ __forceinline__ void store_cols(const CUtensorMap* map, uint32_t tadd
   }
 }
 
+// Where the CTAs of a split key tile leave their dK and dV, from the start of shared
+// memory: per key R + DV floats in 16-byte pieces, swizzled by the key.
 template <int R, int DV>
+struct KeyPartial {
+  static constexpr int PIECES = (R + DV) / 4, ROW = (PIECES + 7) / 8 * 8;
+  static constexpr int BYTES = kKeys * ROW * 16;
+  __device__ static int piece(int key, int c) { return (key * ROW + (c ^ (key & 7))) * 16; }
+};
+
+// W TMEM columns of this thread's key as pieces c0 .. of its partial.
+template <int R, int DV, int W>
+__device__ __forceinline__ void put_partial(uint32_t taddr, unsigned char* smem, int key, int c0) {
+  uint32_t w[W];
+  tmem_ld_n<W>(taddr, w);
+#pragma unroll
+  for (int c = 0; c < W / 4; ++c)
+    *reinterpret_cast<uint4*>(smem + KeyPartial<R, DV>::piece(key, c0 + c)) =
+        make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+}
+
+// This CTA's share of the tile's keys (rank, rank + C, ...) summed over the CTAs
+// that have tiles (bit c of `have`), in their order, and written out by the 512
+// softmax threads.
+template <int R, int DV, int C>
+__device__ __forceinline__ void sum_split(const BackwardParams& p, unsigned char* smem, int rank, uint32_t have, int key0,
+                                          size_t plane, int tid) {
+  using K = KeyPartial<R, DV>;
+  constexpr int U = 8 / C;
+  const int n = (min(kKeys, p.S - key0) - rank + C - 1) / C * K::PIECES;
+  const uint32_t base = smem_addr(smem);
+  for (int q0 = tid; q0 < n; q0 += 512 * U) {
+    float4 y[U][C];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = min(q0 + 512 * u, n - 1);
+      const uint32_t at = base + K::piece(rank + q / K::PIECES * C, q % K::PIECES);
+#pragma unroll
+      for (int c = 0; c < C; ++c) y[u][c] = ld_cluster_f32x4(cluster_addr(at, c));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = q0 + 512 * u, c4 = q % K::PIECES;
+      if (q >= n) continue;
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        if ((have >> c) & 1u) {
+          a.x += y[u][c].x;
+          a.y += y[u][c].y;
+          a.z += y[u][c].z;
+          a.w += y[u][c].w;
+        }
+      }
+      const size_t row = plane * p.S + key0 + rank + q / K::PIECES * C;
+      if (c4 < R / 4) {
+        a = make_float4(a.x * p.scale, a.y * p.scale, a.z * p.scale, a.w * p.scale);
+        *reinterpret_cast<float4*>(p.dk + row * R + 4 * c4) = a;
+      } else {
+        *reinterpret_cast<float4*>(p.dv + row * DV + 4 * c4 - R) = a;
+      }
+    }
+  }
+}
+
+// SPLIT: the CTAs of a cluster share a key tile's query tiles and add up their dK
+// and dV through distributed shared memory at the end; for launches of so few key
+// tiles that SMs would stay idle (choose_split).
+template <int R, int DV, bool SPLIT>
 __global__ void __launch_bounds__(kTcBound, 1)
 bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   using C = TCfg<R, DV>;
@@ -262,15 +330,22 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   const int S = p.S, G = p.Hq / p.Hkv;
   const int n_kt = (S + kKeys - 1) / kKeys;
   const int n_qt = (S + kQT - 1) / kQT;
-  // CTA order: (sequence, kv head) major, the key tiles with most work first
-  const int j = static_cast<int>(blockIdx.x % n_kt);
-  const int bg = static_cast<int>(blockIdx.x / n_kt);
+  // CTA order: (sequence, kv head) major, so that the CTAs at work read the same
+  // queries, or key tile major where all queries stay in L2 anyway; the key tiles with
+  // most work first
+  const uint32_t work = SPLIT ? blockIdx.x / p.split : blockIdx.x;
+  const int rank = SPLIT ? static_cast<int>(blockIdx.x % p.split) : 0;   // = the rank in the cluster
+  const int j = static_cast<int>(p.tile_major ? work / (p.B * p.Hkv) : work % n_kt);
+  const int bg = static_cast<int>(p.tile_major ? work % (p.B * p.Hkv) : work / n_kt);
   const int b = bg / p.Hkv, g = bg % p.Hkv;
   const int i0 = p.causal ? j : 0;     // kKeys == kQT: query tiles i >= j see key tile j
   const int per_head = n_qt - i0;
-  const int n_tiles = G * per_head;
-  auto tile_head = [&](int t) { return g * G + t / per_head; };
-  auto tile_q = [&](int t) { return i0 + t % per_head; };
+  // this CTA's tiles: t0 .. t0 + n_tiles - 1 of the key tile's, counted from t0
+  const int all_tiles = G * per_head;
+  auto first_tile = [&](int c) { return SPLIT ? all_tiles * c / p.split : 0; };
+  const int t0 = first_tile(rank), n_tiles = SPLIT ? first_tile(rank + 1) - t0 : all_tiles;
+  auto tile_head = [&](int t) { return g * G + (t0 + t) / per_head; };
+  auto tile_q = [&](int t) { return i0 + (t0 + t) % per_head; };
   // half tile u = 2 t + h lives in slot u % NSLOT, its (u / NSLOT)-th use of the slot
   auto slot_of = [](int t, int h) { return (2 * t + h) % C::NSLOT; };
   auto slot_par = [](int t, int h) { return static_cast<uint32_t>(((2 * t + h) / C::NSLOT) & 1); };
@@ -312,7 +387,9 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == kWarpTma) {
+  if (SPLIT && n_tiles == 0) {
+    // fewer tiles than CTAs: this one only takes its share of the sums below
+  } else if (warp == kWarpTma) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       const int kv_plane = b * p.Hkv + g;
@@ -498,7 +575,14 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     }
     // dK of the CTA's keys (these warps are done before the softmax warps are)
     const int key0 = j * kKeys + w4 * 32;
-    if (mbar_wait_warp(acc_full, 0, p.err) && key0 < S) {
+    if (SPLIT) {
+      if (mbar_wait_warp(acc_full, 0, p.err)) {
+        tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < R; c0 += C::DQ_W)
+          put_partial<R, DV, C::DQ_W>(tmem + C::T_DK + c0 + lane_off, smem, w4 * 32 + lane, c0 / 4);
+      }
+    } else if (mbar_wait_warp(acc_full, 0, p.err) && key0 < S) {
       tc_fence_after();
       store_cols<R, C::DQ_W>(&maps.dk, tmem + C::T_DK + lane_off, smem + C::OFF_SL + kWarpDq * 4096 + w4 * 8192, p.scale, 0, key0,
                              b * p.Hkv + g, lane);
@@ -590,12 +674,30 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     // tiles are free: every product has read them
     const int key0 = j * kKeys + (warp & 3) * 32, x0 = 32 * (warp >> 2);
     if (ok) ok = mbar_wait(acc_full, 0, p.err);
-    if (__all_sync(0xffffffffu, ok) && key0 < S && x0 < DV) {
+    if (SPLIT) {
+      if (__all_sync(0xffffffffu, ok) && x0 < DV) {
+        tc_fence_after();
+        put_partial<R, DV, 32>(tmem + C::T_DV + x0 + lane_off, smem, kt, (R + x0) / 4);
+      }
+    } else if (__all_sync(0xffffffffu, ok) && key0 < S && x0 < DV) {
       tc_fence_after();
       store_cols<32, 32>(&maps.dv, tmem + C::T_DV + x0 + lane_off, smem + C::OFF_SL + warp * 4096, 1.f, x0, key0,
                          b * p.Hkv + g, lane);
     }
     if (lane == 0) bulk_wait_read_all();
+  }
+  if constexpr (SPLIT) {
+    static_assert(KeyPartial<R, DV>::BYTES <= C::OFF_DQ, "partials over K, V, the ring and the dS tiles");
+    cluster_sync();
+    if (warp < kWarpDq) {
+      uint32_t have = 0;
+      for (int c = 0; c < p.split; ++c) have |= (first_tile(c + 1) > first_tile(c) ? 1u : 0u) << c;
+      const size_t plane = static_cast<size_t>(b) * p.Hkv + g;
+      if (p.split == 2) sum_split<R, DV, 2>(p, smem, rank, have, j * kKeys, plane, tid);
+      else if (p.split == 4) sum_split<R, DV, 4>(p, smem, rank, have, j * kKeys, plane, tid);
+      else sum_split<R, DV, 8>(p, smem, rank, have, j * kKeys, plane, tid);
+    }
+    cluster_sync();  // no CTA leaves while others read its shared memory
   }
   tc_fence_before();
   __syncthreads();
@@ -603,6 +705,35 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemColsTc);
   }
+}
+
+// CTAs per key tile: the number with the least estimated time, in units of one
+// tile's (1.6 us at r = 32): a CTA costs 5 for set-up and epilogue, 2 more if
+// split; causal launches (CTAs of many sizes, the largest first) take the longer of
+// their heaviest CTA and the mean of the SMs, and half a set-up more where a split
+// needs a second CTA on an SM; others whole waves.  A CTA keeps at least two of its
+// key tile's query tiles.  Measured without and with the split: 16/2 heads, r=64,
+// d_v=128, B=3, S=138 41 us -> 16; r=32, B=1, S=2000 206 -> 59; r=128, S=500 117 -> 28;
+// 32/8 heads, r=32, S=300 26 -> 16, S=1531 87 -> 53; but 12 heads, r=16, d_v=64, S=1024
+// 17.4 -> 21.1 with two CTAs a key tile (192 on 152 SMs), so that one is not split.
+int choose_split(const BackwardParams& p, long long grid) {
+  const int n_qt = (p.S + kQT - 1) / kQT;
+  const double heaviest = static_cast<double>(p.Hq / p.Hkv) * n_qt;   // the first key tile's
+  const double total = heaviest * grid * (p.causal ? (n_qt + 1) / (2.0 * n_qt) : 1.0);
+  int best = 1;
+  double least = 0;
+  for (int c = 1; c <= kMaxSplit; c *= 2) {
+    if (c > 1 && heaviest < 2 * c) break;
+    const double fixed = c > 1 ? 7 : 5, one = heaviest / c + fixed;
+    const double mean = (total + grid * c * fixed) / p.num_sms;
+    const double t = p.causal ? std::max(one, mean) + (c > 1 && grid * c > p.num_sms ? fixed / 2 : 0)
+                              : std::ceil(static_cast<double>(grid) * c / p.num_sms) * one;
+    if (c == 1 || t < 0.95 * least) {
+      best = c;
+      least = t;
+    }
+  }
+  return best;
 }
 
 template <int R, int DV>
@@ -617,13 +748,18 @@ cudaError_t launch_tc(const BackwardParams& p, cudaStream_t stream) {
       !make_map(&maps.dk, p.dk, R, p.S, p.B * p.Hkv, C::DQ_W, 32, C::DQ_SW, true) ||
       !make_map(&maps.dv, p.dv, DV, p.S, p.B * p.Hkv, 32, 32, 128, true))
     return cudaErrorInvalidValue;
-  auto kern = bwd_tc_kernel<R, DV>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-  if (e != cudaSuccess) return e;
   const long long n_kt = (p.S + kKeys - 1) / kKeys;
   const long long grid = static_cast<long long>(p.B) * p.Hkv * n_kt;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return launch_pdl(kern, dim3(static_cast<unsigned>(grid)), dim3(kTcThreads), C::SMEM, stream, maps, p);
+  BackwardParams pp = p;
+  pp.split = choose_split(p, grid);
+  // Q and dO of all heads within about 48 MB of L2
+  pp.tile_major = static_cast<long long>(p.B) * p.Hq * p.S * (R + DV) * 2 <= (48LL << 20);
+  auto kern = pp.split > 1 ? bwd_tc_kernel<R, DV, true> : bwd_tc_kernel<R, DV, false>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  if (e != cudaSuccess) return e;
+  return launch_pdl_cluster(kern, dim3(static_cast<unsigned>(grid * pp.split)), dim3(kTcThreads), C::SMEM, stream,
+                            pp.split, maps, pp);
 }
 
 template <int R>

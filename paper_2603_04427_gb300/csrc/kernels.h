@@ -143,6 +143,9 @@ struct BackwardParams {
   int B, Hq, Hkv, S, S_pad, R, DV;
   int causal;
   float scale;
+  int num_sms;
+  int split;          // CTAs (of one cluster) per key tile, set by the launcher
+  int tile_major;     // CTA order: key tile, then (sequence, kv head); set by the launcher
 };
 
 // Rows of the backward's per-row statistics: S rounded up to 128.

@@ -177,36 +177,6 @@ __device__ __forceinline__ void split_bf16(float2 x, uint32_t& hi, uint32_t& lo)
   lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// ---------------------------------------------------------------- clusters
-constexpr int kMaxSplit = 8;  // CTAs of a cluster
-
-// Barrier of all threads of the cluster; shared-memory writes before it are
-// visible to reads after it in every CTA.
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile(
-      "barrier.cluster.arrive.release.aligned;\n\t"
-      "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address of this CTA's shared-memory address in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
-  uint32_t a;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
-  float x;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(addr) : "memory");
-  return x;
-}
-__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
-  float4 x;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
-               : "r"(addr)
-               : "memory");
-  return x;
-}
-
 // Where the CTAs of a split pair leave their partial results, from the start of
 // shared memory: O of both tiles in fp32 ([row][d_v], the 16-byte pieces of a row
 // swizzled by the row), then max and sum per row, then weights of merge_split.

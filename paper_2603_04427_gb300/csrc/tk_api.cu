@@ -220,6 +220,7 @@ tk_status tk_attn_backward(const void* q, const void* k, const void* v, const vo
   p.B = batch; p.Hq = h_q; p.Hkv = h_kv; p.S = seq; p.R = r; p.DV = d_v;
   p.causal = causal != 0;
   p.scale = scale;
+  p.num_sms = dev.num_sms;
   int uns = 0;
   cudaError_t e = tk::launch_backward(p, static_cast<cudaStream_t>(stream), &uns);
   if (uns) return fail(TK_ERR_UNSUPPORTED, "backward: no kernel for r=%d d_v=%d", r, d_v);
