@@ -40,9 +40,12 @@
 // softmaxes run, then both wait (7B shape: 754 us a prompt pass against 640).
 // That warp must then be quick: one election per four products and warp-uniform
 // waits.  K and V leave the ring separately (K after its scores, V after its
-// P V products), which a 2-stage ring (r = 128) needs most: B=2, H=32, S=8192,
-// d_v = 128, causal, kernel time before and after both: r=16 625 -> 598 us, r=32
-// 575 -> 563, r=64 617 -> 585, r=128 963 -> 706.
+// P V products), which a 2-stage ring (r = 128) needs most.  The TMA warp sets the
+// barriers up and issues its first loads before the CTA's other set-up is done, and
+// the output leaves by TMA stores: about 5 us of a CTA's time are set-up, first loads
+// and epilogue.  Kernel time before and after these, B=2, H=32, S=8192, d_v = 128,
+// causal: r=16 625 -> 573 us, r=32 575 -> 542, r=64 617 -> 562, r=128 963 -> 674 (of
+// it K / V release and the MMA warp: 598, 563, 585, 706).
 //
 // TMEM columns: [0,128) S_A, [128,256) S_B (each: fp32 scores, the first 64
 // columns later hold P as packed bf16 pairs), [256,384) O_A, [384,512) O_B.
@@ -319,8 +322,10 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   const int kv_plane = b * p.Hkv + h / (p.Hq / p.Hkv);
   const int qa = 2 * tp, qb = 2 * tp + 1;
   const bool has_b = qb < n_qt;
-  // set-up that reads no global memory runs while the previous kernel finishes
-  if (tid == 0) {
+  // set-up that reads no global memory runs while the previous kernel finishes.  The
+  // TMA warp sets the barriers up itself, so that its first loads need not wait for
+  // the other warps and the TMEM allocation.
+  if (warp == 8 && lane == 0) {
     mbar_init(q_full, 1);
     for (int s = 0; s < NST; ++s) {
       mbar_init(&k_full[s], 1);
@@ -338,11 +343,14 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     fence_barrier_init();
   }
   if (warp == 8) {
+    __syncwarp();
     if (lane == 0) {
       prefetch_map(&maps.q);
       prefetch_map(&maps.k);
       prefetch_map(&maps.v);
     }
+  }
+  if (warp == 9) {
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
@@ -375,12 +383,6 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     n_kv = j1 - j0;
   }
 
-  __syncthreads();
-  // after the barrier, so that every CTA of this grid holds its TMEM before a
-  // CTA of the next kernel can ask for some
-  pdl_trigger();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
 
   // In cached mode the tile holding the context's end is "relayed": it lands on
   // c_full, the TMA warp zeroes its value rows past the context (the cache may
@@ -406,6 +408,15 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     return true;
   };
 
+  // everyone's set-up is done, and every CTA of this grid holds its TMEM before a
+  // CTA of the next kernel can ask for some
+  auto set_up = [&]() -> uint32_t {
+    __syncthreads();
+    pdl_trigger();
+    tc_fence_after();
+    return *tmem_slot;
+  };
+  uint32_t tmem;
   if (warp == 8) {
     // ------------------------------------------------------------------ TMA producer
     // K/V maps are [planes][rows][width]: plane b*Hkv + g with rows = S (plain) or
@@ -482,12 +493,16 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       }
       return true;
     };
-    for (int j = 0; j < n_kv; ++j) {
-      if (!issue(j)) break;
+    const bool ok = n_kv == 0 || issue(0);
+    __syncwarp();
+    tmem = set_up();
+    for (int j = 0; ok && j < n_kv; ++j) {
+      if (j > 0 && !issue(j)) break;
       if (relayed(j) && !finish(j)) break;
     }
   } else if (warp == 9) {
     // ------------------------------------------------------------------ MMA issuer
+    tmem = set_up();
     {
       // descriptors of Q tile A and of the K / V tiles of stage 0; other
       // stages and K steps are start-address offsets from these
@@ -556,6 +571,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     }
   } else {
     // ------------------------------------------------------------------ softmax warps
+    tmem = set_up();
     const int x = warp >> 2;                   // 0: tile A, 1: tile B
     const int nx = x == 0 ? n_a : n_b;
     const int qt = x == 0 ? qa : qb;
@@ -762,7 +778,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
+  if (warp == 9) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
