@@ -141,7 +141,11 @@ tk_status tk_kv_append(const tk_cache_desc* desc, void* k_cache, void* v_cache, 
  * Shapes: r in {16, 32, 64, 128}, d_v in {64, 128}, h_q % h_kv == 0,
  * seq >= 0 (seq == 0 is a no-op).  Scores and the weighted sum accumulate
  * in fp32 on the tensor cores; the softmax weights enter the second
- * product rounded to bf16.                                                  */
+ * product rounded to bf16.  Launches of few query tiles split the keys over
+ * a thread-block cluster (another order of the same sums; results are
+ * deterministic for a given shape).  Launched with programmatic dependent
+ * launch (see tk_attn_decode), as are tk_attn_forward, tk_attn_backward and
+ * tk_attn_prefill_cached.                                                   */
 tk_status tk_attn_prefill(const void* q, const void* k, const void* v, void* out,
                           int32_t out_dtype, int32_t batch, int32_t h_q, int32_t h_kv,
                           int32_t seq, int32_t r, int32_t d_v, float scale, int32_t causal,
@@ -178,7 +182,7 @@ size_t tk_backward_workspace_size(int32_t batch, int32_t h_q, int32_t seq);
  * The products run on the tensor cores with bf16 operands (P and dS rounded
  * to bf16) and fp32 accumulation (tcgen05, accumulators in tensor memory);
  * dq is accumulated across key tiles with fp32 reduce-adds, so its
- * low bits may vary run to run.  Two launches (preprocessing, gradients).    */
+ * low bits may vary run to run (dk and dv are summed in a fixed order).  Two launches (preprocessing, gradients).    */
 tk_status tk_attn_backward(const void* q, const void* k, const void* v, const void* out,
                            const void* d_out, const float* lse, float* dq, float* dk, float* dv,
                            void* workspace, size_t workspace_bytes, int32_t batch, int32_t h_q,
