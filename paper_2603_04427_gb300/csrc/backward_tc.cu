@@ -44,7 +44,8 @@
 // S=8192, r=32, d_v=128, causal, preprocessing included): dQ read back by warps of
 // its own instead of by the softmax warps (1987 -> 1743 us), sixteen softmax warps
 // with 80 registers instead of eight with 168 and dK / dV through TMA stores
-// (1655), the statistics apart from the tiles and two staging places for dQ (1608).
+// (1655), the statistics apart from the tiles and two staging places for dQ (1608),
+// warp-uniform waits of the softmax warps (1601).
 // One product of N = 128 for both halves' S^T and dP^T needs fewer reads of K and
 // V, but the halves then run in step and wait together: 1820 us.
 //
@@ -603,10 +604,9 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
     for (int t = 0; t < n_tiles; ++t) {
       const int sl = slot_of(t, h), buf = t % NDS;
       if (ok) {
-        ok = mbar_wait(&s_full[h], t & 1, p.err) && mbar_wait(&sl_full[sl], slot_par(t, h), p.err);
+        ok = mbar_wait_warp(&s_full[h], t & 1, p.err) && mbar_wait_warp(&sl_full[sl], slot_par(t, h), p.err);
         // (with one dS tile its buffer is asked for as late as possible, below)
-        if (NDS > 1 && ok && t >= NDS) ok = mbar_wait(&ds_free[buf], ((t / NDS) - 1) & 1, p.err);
-        ok = __all_sync(0xffffffffu, ok);
+        if (NDS > 1 && ok && t >= NDS) ok = mbar_wait_warp(&ds_free[buf], ((t / NDS) - 1) & 1, p.err);
       }
       if (ok) {
         tc_fence_after();
@@ -644,10 +644,8 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
           // P^T_h may overwrite the previous tile's only once its dV product has read
           // it, dS^T_h its buffer's last tile once its dK and dQ products have
           if (!(c & 1) && t > 0 && (C::P_OWN || NDS == 1)) {
-            bool okp = true;
-            if (C::P_OWN) okp = mbar_wait(&p_free[h], (t - 1) & 1, p.err);
-            if (NDS == 1) okp = mbar_wait(&ds_free[0], (t - 1) & 1, p.err) && okp;
-            if (!__all_sync(0xffffffffu, okp)) ok = false;
+            if (C::P_OWN && !mbar_wait_warp(&p_free[h], (t - 1) & 1, p.err)) ok = false;
+            if (NDS == 1 && !mbar_wait_warp(&ds_free[0], (t - 1) & 1, p.err)) ok = false;
           }
           // over scores that this warp itself has read, where P^T has no columns of its own
           tmem_st8(tP + (C::P_OWN ? 8 * c : 32 * (c >> 1) + 8 * (c & 1)), pk);

@@ -44,8 +44,9 @@
 // barriers up and issues its first loads before the CTA's other set-up is done, and
 // the output leaves by TMA stores: about 5 us of a CTA's time are set-up, first loads
 // and epilogue.  Kernel time before and after these, B=2, H=32, S=8192, d_v = 128,
-// causal: r=16 625 -> 573 us, r=32 575 -> 542, r=64 617 -> 562, r=128 963 -> 674 (of
-// it K / V release and the MMA warp: 598, 563, 585, 706).
+// causal: r=16 625 -> 568 us, r=32 575 -> 536, r=64 617 -> 556, r=128 963 -> 671 (of
+// it K / V release and the MMA warp: 598, 563, 585, 706; the softmax warps' waits made
+// warp-uniform: 573, 542, 562, 674 before it).
 //
 // TMEM columns: [0,128) S_A, [128,256) S_B (each: fp32 scores, the first 64
 // columns later hold P as packed bf16 pairs), [256,384) O_A, [384,512) O_B.
@@ -583,8 +584,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     float m_used = -INFINITY, l = 0.f;
     bool ok = nx > 0;
     for (int j = 0; j < nx; ++j) {
-      ok = mbar_wait(&s_full[x], j & 1, p.err);
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      if (!(ok = mbar_wait_warp(&s_full[x], j & 1, p.err))) break;
       tc_fence_after();
       const int kv0 = (j0 + j) * kBN;
       const bool masked = (p.causal && kv0 + kBN - 1 > L0 + qt * kBM) || (kv0 + kBN > kv_len);
