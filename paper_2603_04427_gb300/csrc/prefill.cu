@@ -183,7 +183,9 @@ __device__ __forceinline__ void split_bf16(float2 x, uint32_t& hi, uint32_t& lo)
 
 // Where the CTAs of a split pair leave their partial results, from the start of
 // shared memory: O of both tiles in fp32 ([row][d_v], the 16-byte pieces of a row
-// swizzled by the row), then max and sum per row, then weights of merge_split.
+// swizzled by the row), then max and sum per row, then weights of merge_split.  The
+// max is -inf where the CTA saw no key of the row, and NaN where a score was NaN.
+constexpr float kNoKeys = -1.f;   // weight of a CTA without keys of the row, whose O may be anything
 template <int DV>
 struct Partial {
   static constexpr int STAT = 2 * kBM * DV * 4;                     // [tile][max, sum][row]
@@ -218,11 +220,13 @@ __device__ __forceinline__ void merge_split(const PrefillParams& p, unsigned cha
     for (int c = 0; c < C; ++c) mx = fmaxf(mx, m[c]);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-      m[c] = m[c] == -INFINITY ? 0.f : fast_exp2(m[c] - mx);  // -inf: no key of the row there
-      if (m[c] != 0.f) sum += l[c] * m[c];
+      m[c] = m[c] == -INFINITY ? kNoKeys : fast_exp2(m[c] - mx);
+      if (m[c] != kNoKeys) sum += l[c] * m[c];
     }
+    // (a CTA with the largest max has a sum of at least 1; 0: every visible score is -inf)
+    const float none = sum == 0.f ? NAN : kNoKeys;
 #pragma unroll
-    for (int c = 0; c < C; ++c) weight[tid * C + c] = m[c] / sum;
+    for (int c = 0; c < C; ++c) weight[tid * C + c] = m[c] == kNoKeys ? none : m[c] / sum;
   }
   asm volatile("bar.sync 1, 256;" ::: "memory");
   for (int q0 = tid; q0 < rows * PIECES; q0 += 256 * U) {
@@ -244,7 +248,7 @@ __device__ __forceinline__ void merge_split(const PrefillParams& p, unsigned cha
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        if (w[u][c] != 0.f) {  // what a CTA without keys of the row holds may be anything
+        if (w[u][c] != kNoKeys) {  // (a weight of 0 counts: 0 * NaN is NaN, as in one CTA's sums)
           o.x += w[u][c] * y[u][c].x;
           o.y += w[u][c] * y[u][c].y;
           o.z += w[u][c] * y[u][c].z;
@@ -691,7 +695,8 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       }
       float* stat = reinterpret_cast<float*>(smem + Partial<DV>::STAT) + x * 2 * kBM;
       const int i = tid & 127;
-      stat[i] = ok && nx > 0 ? m_used : -INFINITY;
+      // (the running max passes NaN scores by, the sum does not)
+      stat[i] = ok && nx > 0 ? (l == l ? m_used : l) : -INFINITY;
       stat[kBM + i] = l;
       if (ok && nx > 0 && qt * kBM + (warp & 3) * 32 < p.S) {
         tc_fence_after();

@@ -91,3 +91,35 @@ def test_chunk_split(hq, hkv, S, lens, r, dv, page, keys):
             ref = oa.attention_head(f64(q[b, h]), kq[b, h // G, :n + S], f64(v[b, h // G, :n + S]),
                                     1 / math.sqrt(r), causal_offset=n)
             parity(f64(out[b, h]), ref, what=f"split chunk b={b} h={h} {keys} r={r} page={page}")
+
+
+@pytest.mark.parametrize("where", ["share", "diagonal", "value"])
+def test_a_nan_is_not_lost_in_the_merge(where):
+    """Rows that see a NaN key or value are NaN whichever CTA of the cluster sees it, and only those.
+
+    S = 3100, one head: 13 pairs of query tiles over clusters of 8 CTAs, so the first pair's
+    two kv tiles lie in CTAs 3 and 7: of CTA 7's keys row 128 sees key 128 alone.  A value
+    whose weight underflows to 0 is NaN times 0 in one CTA's sums, so it is in the merge.
+    """
+    require_gpu()
+    S, r, dv = 3100, 32, 64
+    q = inputs.normal_bf16((1, 1, S, r), 101, device="cuda")
+    k = inputs.normal_bf16((1, 1, S, r), 102, device="cuda")
+    v = inputs.normal_bf16((1, 1, S, dv), 103, device="cuda")
+    if where == "share":
+        first = 128
+        k[0, 0, first] = float("nan")
+    elif where == "diagonal":
+        first = 2943     # the last row of a tile
+        k[0, 0, first, 3] = float("nan")
+    else:
+        # keys 0 .. 127 score 400 below the others: e^-400 is 0 in fp32
+        first = 0
+        q[..., 0], k[..., 0], k[0, 0, :128, 0] = 40.0, 10.0, -46.5
+        v[0, 0, 5] = float("nan")
+    out = torch.empty((1, 1, S, dv), device="cuda")
+    tb.tk_attn_prefill(q, k, v, out)
+    assert tb.tk_get_device_error() == 0
+    bad = torch.isnan(out[0, 0]).any(1)
+    assert bad[first:].all(), f"rows {torch.nonzero(~bad[first:])[:4].flatten().tolist()} past {first} are finite"
+    assert not bad[:first].any()
