@@ -127,8 +127,7 @@ struct TCfg {
   static constexpr int OFF_DQ = OFF_DS + NDS * DSB;
   static constexpr int OFF_ST = OFF_DQ + DQB;
   static constexpr int OFF_BAR = OFF_ST + NSLOT * STATS;
-  // at least 116 KB so that one CTA (and its 512 TMEM columns) sits on an SM alone
-  static constexpr int SMEM = std::max(OFF_BAR + 256 + 1024, 116 * 1024);
+  static constexpr int SMEM = std::max(OFF_BAR + 256 + 1024, kOneCtaSmem);
   static_assert(OFF_BAR + 256 + 1024 <= 227 * 1024, "shared memory");
   static_assert(OFF_DQ - OFF_SL >= kWarpDq * 4096 + 4 * 8192, "staging places of the epilogue");
   // TMEM columns

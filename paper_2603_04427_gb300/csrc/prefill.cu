@@ -131,7 +131,8 @@ struct PCfg {
   static constexpr int OFF_SC = OFF_K + NST * STAGE;
   static constexpr int OFF_BAR = OFF_SC + NST * SCB;
   static constexpr int SMEM = OFF_BAR + 256 + 1024;      // + slack to align the base to 1 KB
-  static_assert(SMEM <= 227 * 1024, "shared memory");
+  static constexpr int SMEM_SPLIT = std::max(SMEM, kOneCtaSmem);   // CTAs of a cluster
+  static_assert(SMEM_SPLIT <= 227 * 1024, "shared memory");
   static constexpr uint32_t IDESC_S = instr_desc(kBM, kBN, false);
   static constexpr uint32_t IDESC_O = instr_desc(kBM, DV, true);
 };
@@ -920,7 +921,7 @@ cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   if (grid > 0x7fffffffL) return cudaErrorInvalidConfiguration;
   pp.split = choose_split(p, grid);
   auto kern = pp.split > 1 ? prefill_kernel<R, DV, KF, true> : prefill_kernel<R, DV, KF, false>;
-  const int smem = C::SMEM;
+  const int smem = pp.split > 1 ? C::SMEM_SPLIT : C::SMEM;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   if constexpr (KF != kKeyBF16) {

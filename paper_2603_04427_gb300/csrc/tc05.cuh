@@ -274,6 +274,13 @@ constexpr uint32_t instr_desc(int M, int N, bool b_mn_major, bool a_mn_major = f
 
 // ---------------------------------------------------------------- clusters
 constexpr int kMaxSplit = 8;  // CTAs of a cluster
+// Shared memory that only one CTA of an SM's 228 KB can hold (each takes 1 KB more).
+// A CTA of a cluster keeps all TMEM columns until it has met its peers at the cluster's
+// barrier, and neither that barrier nor tcgen05.alloc is a bounded wait: with two such
+// CTAs on one SM, the second one's allocation could wait for the first and the first,
+// at the barrier, for a peer that waits in turn for a CTA like it.
+constexpr int kOneCtaSmem = 116 * 1024;
+static_assert(2 * (kOneCtaSmem + 1024) > 228 * 1024, "one CTA an SM");
 
 // Barrier of all threads of the cluster; shared-memory writes before it are
 // visible to reads after it in every CTA.
