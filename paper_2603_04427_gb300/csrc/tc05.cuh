@@ -283,8 +283,10 @@ constexpr int kOneCtaSmem = 116 * 1024;
 static_assert(2 * (kOneCtaSmem + 1024) > 228 * 1024, "one CTA an SM");
 
 // Barrier of all threads of the cluster; shared-memory writes before it are
-// visible to reads after it in every CTA.
+// visible to reads after it in every CTA.  The .aligned forms want every lane of
+// the warp together, and callers come from code of single lanes.
 __device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
       "barrier.cluster.wait.acquire.aligned;" ::: "memory");
