@@ -390,6 +390,7 @@ __device__ __forceinline__ void merge_partials(const float* part, const Split& s
 }
 
 __device__ __forceinline__ void merge_sync() {
+  __syncwarp();   // (bar.sync wants the warp's lanes together)
   asm volatile("bar.sync 1, %0;" ::"n"(kMergeWarps * 32) : "memory");
 }
 

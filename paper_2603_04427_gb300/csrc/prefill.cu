@@ -229,6 +229,7 @@ __device__ __forceinline__ void merge_split(const PrefillParams& p, unsigned cha
 #pragma unroll
     for (int c = 0; c < C; ++c) weight[tid * C + c] = m[c] == kNoKeys ? none : m[c] / sum;
   }
+  __syncwarp();   // (bar.sync wants the warp's lanes together)
   asm volatile("bar.sync 1, 256;" ::: "memory");
   for (int q0 = tid; q0 < rows * PIECES; q0 += 256 * U) {
     float4 y[U][C];
