@@ -142,9 +142,11 @@ tk_status tk_kv_append(const tk_cache_desc* desc, void* k_cache, void* v_cache, 
  * seq >= 0 (seq == 0 is a no-op).  Scores and the weighted sum accumulate
  * in fp32 on the tensor cores; the softmax weights enter the second
  * product rounded to bf16.  Launches of few query tiles split the keys over
- * a thread-block cluster (another order of the same sums; results are
- * deterministic for a given shape).  Launched with programmatic dependent
- * launch (see tk_attn_decode), as are tk_attn_forward, tk_attn_backward and
+ * a thread-block cluster, which is another order of the same sums: the low
+ * bits of a sequence's result depend on batch and h_q as well as on its own
+ * shape, and are the same in every call with these.  tk_attn_forward is
+ * never split.  Launched with programmatic dependent launch (see
+ * tk_attn_decode), as are tk_attn_forward, tk_attn_backward and
  * tk_attn_prefill_cached.                                                   */
 tk_status tk_attn_prefill(const void* q, const void* k, const void* v, void* out,
                           int32_t out_dtype, int32_t batch, int32_t h_q, int32_t h_kv,
@@ -220,7 +222,9 @@ tk_status tk_attn_backward(const void* q, const void* k, const void* v, const vo
  * chunk does not fit sets the device error word and is computed over a
  * clamped context.  Cache slots past a sequence's context may hold anything
  * (they are never weighted).  seq_lens[b] == 0 gives the plain causal
- * prefill of the chunk.  Launches in stream order: append, (key widening,)
+ * prefill of the chunk (over bf16 keys, the same bits).  The split of
+ * tk_attn_prefill goes by each sequence's own context: max_seq_len does not
+ * change the result.  Launches in stream order: append, (key widening,)
  * attention.                                                              */
 tk_status tk_attn_prefill_cached(const tk_cache_desc* desc, const void* q, void* k_cache,
                                  void* v_cache, float* k_scale, const int32_t* page_table,

@@ -62,6 +62,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "split.h"
 #include "tc05.cuh"
 
 namespace tk {

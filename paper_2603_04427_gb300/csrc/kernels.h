@@ -104,7 +104,7 @@ struct PrefillParams {
   float scale_log2;
   int num_sms;
   int head_group;  // (b, h) pairs per L2 group, set by the launcher
-  int split;       // CTAs (of one cluster) per query tile pair, set by the launcher
+  int split;       // CTAs of a cluster, which share a query tile pair; set by the launcher
   // cached mode (a chunk of S queries after seq_lens[b] cached tokens):
   // query i of sequence b sits at position seq_lens[b] + i and the keys are
   // the cache's first seq_lens[b] + S tokens (bottom-right causal)

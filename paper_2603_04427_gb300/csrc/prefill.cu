@@ -54,6 +54,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "split.h"
 #include "tc05.cuh"
 #include "widen.cuh"
 
@@ -287,10 +288,10 @@ struct Maps {
 //   warps 4-7: the same for tile B
 //   warp 8: TMA producer (Q tiles once, K/V tiles into an NST-stage ring)
 //   warp 9: MMA issuer
-// SPLIT: the CTAs of a cluster compute the same two query tiles, each over its
-// share of the kv tiles, and merge their partial results through distributed
-// shared memory at the end; for launches of so few query tiles that SMs would stay
-// idle (choose_split).
+// SPLIT: the CTAs of a cluster (all of them, or as many as the sequence has kv tiles
+// for: prefill_shares) compute the same two query tiles, each over its share of the kv
+// tiles, and merge their partial results through distributed shared memory at the end;
+// for launches of so few query tiles that SMs would stay idle (prefill_cluster).
 template <int R, int DV, int KF, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
@@ -382,9 +383,13 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
   int n_b = has_b ? tiles_for(qb) : 0;
   int n_kv = max(n_a, n_b);
   int j0 = 0;  // this CTA's kv tiles: j0 .. j0 + n_kv - 1, counted from j0 below
+  int shares = 1;  // CTAs of the cluster with a share: ranks 0 .. shares - 1
   if constexpr (SPLIT) {
-    j0 = n_kv * rank / p.split;
-    const int j1 = n_kv * (rank + 1) / p.split;
+    shares = prefill_shares(n_kv_all, p.split);
+    // (shares is a power of two; beyond it the two bounds are n_kv)
+    const int lg = __popc(shares - 1);
+    j0 = n_kv * min(rank, shares) >> lg;
+    const int j1 = n_kv * min(rank + 1, shares) >> lg;
     n_a = max(0, min(n_a, j1) - j0);
     n_b = max(0, min(n_b, j1) - j0);
     n_kv = j1 - j0;
@@ -686,7 +691,7 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       const float2 s01 = fadd2(acc[0], acc[1]), s23 = fadd2(acc[2], acc[3]);
       l += (s01.x + s01.y) + (s23.x + s23.y);
     }
-    if constexpr (SPLIT) {
+    if (SPLIT && shares > 1) {
       // Partial result of this CTA (Partial) over the ring and the Q tiles, once both
       // tiles' products and so all loads are complete; max -inf where this CTA had no
       // kv tile for the row.
@@ -721,64 +726,72 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
       // natural-log logsumexp of the row's scaled scores (for the backward):
       // sum_j exp(scale s_j) = 2^m_used * l
       if (p.lse && row < p.S) p.lse[static_cast<size_t>(bh) * p.S + row] = (m_used + log2f(l)) * 0.69314718055994531f;
-      // the whole O row with one TMEM wait (the score registers are free by now)
-      uint32_t o[DV];
-      if constexpr (DV == 128) tmem_ld128(tO + lane_off, o);
-      else tmem_ld64(tO + lane_off, o);
-      // 128-byte column boxes of the warp's 32 rows through shared memory (its part of
-      // the tile's Q, which every score product has read) and TMA stores, rows past
-      // the sequence cut off.  Row stores by thread touch 32 lines each:
-      // B=64, H=32, S=256, r=32, d_v=128 110 us against 104, B=1, 32/8 heads, S=1531
-      // 22.1 against 19.0.
-      unsigned char* stage = smem + C::OFF_Q + x * C::QBA + (warp & 3) * 4096;
-      const int row0 = qt * kBM + (warp & 3) * 32;
-      auto put = [&](int box, auto&& piece, int width) {  // piece(c): 16 bytes c of the row's 128
-        if (box > 0) {
-          if (lane == 0) bulk_wait_read_all();
+      // The whole O row with one TMEM wait (the score registers are free by now).  In a
+      // cluster's kernel, for sequences too short to be split, 64 columns at a time:
+      // half the code beside the merge's, which it otherwise slows down (32/8 heads, 23
+      // tokens after 13000 32.7 us against 33.4; at r = 128 it is the other way round,
+      // 16/2 heads, B=2, 300 after 1000 19.3 against 19.2).
+      constexpr int OW = SPLIT && R < 128 ? 64 : DV;
+#pragma unroll 1
+      for (int x0 = 0; x0 < DV; x0 += OW) {
+        uint32_t o[OW];
+        if constexpr (OW == 128) tmem_ld128(tO + lane_off + x0, o);
+        else tmem_ld64(tO + lane_off + x0, o);
+        // 128-byte column boxes of the warp's 32 rows through shared memory (its part of
+        // the tile's Q, which every score product has read) and TMA stores, rows past
+        // the sequence cut off.  Row stores by thread touch 32 lines each:
+        // B=64, H=32, S=256, r=32, d_v=128 110 us against 104, B=1, 32/8 heads, S=1531
+        // 22.1 against 19.0.
+        unsigned char* stage = smem + C::OFF_Q + x * C::QBA + (warp & 3) * 4096;
+        const int row0 = qt * kBM + (warp & 3) * 32;
+        auto put = [&](int box, auto&& piece, int width) {  // piece(c): 16 bytes c of the row's 128
+          if (box > 0 || x0 > 0) {
+            if (lane == 0) bulk_wait_read_all();
+            __syncwarp();
+          }
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = piece(c);
+          fence_proxy_async_smem();
           __syncwarp();
+          if (lane == 0 && row0 < p.S) {
+            tma_store_3d(&maps.out, stage, x0 + box * width, row0, bh);
+            bulk_commit();
+          }
+        };
+        auto val = [&](int e) { return __uint_as_float(o[e]) * inv; };
+        if (p.out_f32) {
+#pragma unroll
+          for (int i = 0; i < OW / 32; ++i)
+            put(i, [&](int c) {
+              const int e = 32 * i + 4 * c;
+              return make_uint4(__float_as_uint(val(e)), __float_as_uint(val(e + 1)), __float_as_uint(val(e + 2)),
+                                __float_as_uint(val(e + 3)));
+            }, 32);
+        } else {
+#pragma unroll
+          for (int i = 0; i < OW / 64; ++i)
+            put(i, [&](int c) {
+              uint32_t w[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int e = 64 * i + 8 * c + 2 * k;
+                __nv_bfloat162 pr = __floats2bfloat162_rn(val(e), val(e + 1));
+                w[k] = *reinterpret_cast<uint32_t*>(&pr);
+              }
+              return make_uint4(w[0], w[1], w[2], w[3]);
+            }, 64);
         }
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          *reinterpret_cast<uint4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = piece(c);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0 && row0 < p.S) {
-          tma_store_3d(&maps.out, stage, box * width, row0, bh);
-          bulk_commit();
-        }
-      };
-      auto val = [&](int e) { return __uint_as_float(o[e]) * inv; };
-      if (p.out_f32) {
-#pragma unroll
-        for (int i = 0; i < DV / 32; ++i)
-          put(i, [&](int c) {
-            const int e = 32 * i + 4 * c;
-            return make_uint4(__float_as_uint(val(e)), __float_as_uint(val(e + 1)), __float_as_uint(val(e + 2)),
-                              __float_as_uint(val(e + 3)));
-          }, 32);
-      } else {
-#pragma unroll
-        for (int i = 0; i < DV / 64; ++i)
-          put(i, [&](int c) {
-            uint32_t w[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int e = 64 * i + 8 * c + 2 * k;
-              __nv_bfloat162 pr = __floats2bfloat162_rn(val(e), val(e + 1));
-              w[k] = *reinterpret_cast<uint32_t*>(&pr);
-            }
-            return make_uint4(w[0], w[1], w[2], w[3]);
-          }, 64);
       }
       if (lane == 0) bulk_wait_read_all();
     }
     }
   }
-  if constexpr (SPLIT) {
+  if (SPLIT && shares > 1) {
     cluster_sync();
-    if (warp < 8) {
-      if (p.split == 2) merge_split<DV, 2>(p, smem, rank, qa, bh, tid);
-      else if (p.split == 4) merge_split<DV, 4>(p, smem, rank, qa, bh, tid);
+    if (warp < 8 && rank < shares) {
+      if (shares == 2) merge_split<DV, 2>(p, smem, rank, qa, bh, tid);
+      else if (shares == 4) merge_split<DV, 4>(p, smem, rank, qa, bh, tid);
       else merge_split<DV, 8>(p, smem, rank, qa, bh, tid);
     }
     cluster_sync();  // no CTA leaves while others read its shared memory
@@ -865,21 +878,6 @@ __global__ void __launch_bounds__(256) key_widen_kernel(const PrefillParams p, _
 
 // ---------------------------------------------------------------- host side
 
-// CTAs per query tile pair: as many as find an SM each, where the kv tiles saved
-// (about 1 us each) are worth the merge (3 to 4 us), and every CTA keeps three.
-// Not where the row logsumexp is wanted: a training step's forward keeps one order
-// of sums whatever its batch.  Measured, r = 32, d_v = 128, one CTA a pair against
-// split: 32/8 heads, 500 tokens after 8000 82 us -> 51 (two CTAs), 23 after 13000
-// 100 -> 35 (four); 16/8 heads, B=2, 500 after 2000, int8 35 -> 30; but 500 after 500
-// (8 kv tiles) 16.8 -> 18.0 and a prompt of 512 (4) 9.6 -> 12.0.
-int choose_split(const PrefillParams& p, long pairs) {
-  const long kv_tiles = ((p.seq_lens ? p.kv_limit : p.S) + kBN - 1) / kBN;
-  if (p.lse || kv_tiles < 10) return 1;
-  int split = 1;
-  while (2 * split <= kMaxSplit && pairs * 2 * split <= p.num_sms && kv_tiles >= 6 * split) split *= 2;
-  return split;
-}
-
 template <int R, int DV, int KF>
 cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   using C = PCfg<R, DV, KF>;
@@ -920,7 +918,9 @@ cudaError_t launch_t(const PrefillParams& p, cudaStream_t stream) {
   const long n_qt = (p.S + kBM - 1) / kBM;
   const long grid = (n_qt + 1) / 2 * p.B * p.Hq;  // one CTA per query tile pair
   if (grid > 0x7fffffffL) return cudaErrorInvalidConfiguration;
-  pp.split = choose_split(p, grid);
+  // a training step's forward (lse) keeps one order of sums whatever its batch
+  const int kv_tiles = ((p.seq_lens ? p.kv_limit : p.S) + kBN - 1) / kBN;
+  pp.split = p.lse ? 1 : prefill_cluster(grid, kv_tiles, p.num_sms);
   auto kern = pp.split > 1 ? prefill_kernel<R, DV, KF, true> : prefill_kernel<R, DV, KF, false>;
   const int smem = pp.split > 1 ? C::SMEM_SPLIT : C::SMEM;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -273,7 +273,6 @@ constexpr uint32_t instr_desc(int M, int N, bool b_mn_major, bool a_mn_major = f
 }
 
 // ---------------------------------------------------------------- clusters
-constexpr int kMaxSplit = 8;  // CTAs of a cluster
 // Shared memory that only one CTA of an SM's 228 KB can hold (each takes 1 KB more).
 // A CTA of a cluster keeps all TMEM columns until it has met its peers at the cluster's
 // barrier, and neither that barrier nor tcgen05.alloc is a bounded wait: with two such

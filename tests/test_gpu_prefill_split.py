@@ -15,6 +15,7 @@ import pytest
 import torch
 
 from _helpers import f64, parity, parity_bf16, require_gpu
+from _split import prefill_pairs, rules, tiles
 from oracle import attention as oa
 from oracle import cache as oc
 from paper_2603_04427_gb300 import binding as tb
@@ -123,3 +124,50 @@ def test_a_nan_is_not_lost_in_the_merge(where):
     bad = torch.isnan(out[0, 0]).any(1)
     assert bad[first:].all(), f"rows {torch.nonzero(~bad[first:])[:4].flatten().tolist()} past {first} are finite"
     assert not bad[:first].any()
+
+
+@pytest.mark.parametrize("B,hq,hkv,S,lens,r,dv,page,keys,shares", [
+    (1, 4, 2, 300, [500], 32, 128, 0, "bf16", 1),         # one CTA of eight has work
+    (1, 4, 2, 300, [0], 32, 128, 0, "bf16", 1),           # the plain prefill
+    (1, 2, 1, 2000, [0], 16, 64, 0, "bf16", 4),           # the plain prefill, split itself
+    (1, 4, 4, 200, [1400], 64, 64, 64, "bf16", 4),        # four of eight
+    (2, 8, 2, 130, [3000, 77], 32, 128, 16, "int8", 8),   # eight beside one, in one launch
+    (1, 4, 1, 100, [600], 128, 128, 0, "int4", 1),
+])
+def test_the_bound_does_not_change_the_result(B, hq, hkv, S, lens, r, dv, page, keys, shares):
+    """A loose max_seq_len launches clusters of up to eight CTAs over short contexts: each
+    sequence is split by its own length, so the bits are those of a tight bound (and, for an
+    empty cache, of the plain prefill)."""
+    require_gpu()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tight, loose = max(lens) + S, 16384
+    own = rules().prefill_cluster(prefill_pairs(B, hq, S), tiles(tight), sms)
+    assert own == shares and rules().prefill_cluster(prefill_pairs(B, hq, S), tiles(loose), sms) > min(shares, 4)
+    g = dict(device="cuda")
+    kw = dict(k_int8=keys == "int8", k_int4=keys == "int4")
+    if page:
+        table, n = inputs.paged_layout([loose] * B, page, seed=111)
+        cache = tb.ThinKeyCache.allocate(B, hq, hkv, r, dv, page_size=page, num_pages=n, page_table=table, **kw)
+    else:
+        cache = tb.ThinKeyCache.allocate(B, hq, hkv, r, dv, capacity=loose, **kw)
+    L = max(lens)
+    q, k, v = (inputs.normal_bf16(s, 112 + i, **g) for i, s in enumerate(
+        ((B, hq, S, r), (B, hkv, L + S, r), (B, hkv, L + S, dv))))
+    kn, vn = k[:, :, L:].contiguous(), v[:, :, L:].contiguous()
+    if L:
+        tb.tk_kv_append(cache, k[:, :, :L].contiguous(), v[:, :, :L].contiguous(),
+                        torch.zeros(B, dtype=torch.int32, **g))
+    sl = torch.tensor(lens, dtype=torch.int32, **g)
+    outs = []
+    for bound in (tight, 4096, loose):
+        out = torch.full((B, hq, S, dv), float("nan"), **g)
+        tb.tk_attn_prefill_cached(cache, q, kn, vn, sl, bound, out)
+        assert tb.tk_get_device_error() == 0
+        outs.append(out)
+    if L == 0:
+        out = torch.full((B, hq, S, dv), float("nan"), **g)
+        tb.tk_attn_prefill(q, kn, vn, out)
+        outs.append(out)
+    assert torch.isfinite(outs[0]).all()
+    for out in outs[1:]:
+        assert torch.equal(outs[0], out)
