@@ -20,6 +20,8 @@ from dataclasses import dataclass
 
 import torch
 
+from . import build
+
 TK_OK, TK_ERR_INVALID_ARG, TK_ERR_UNSUPPORTED, TK_ERR_WORKSPACE, TK_ERR_CUDA, TK_ERR_DEVICE = range(6)
 TK_BF16, TK_F32, TK_I8, TK_I4 = 0, 1, 2, 3
 
@@ -46,7 +48,7 @@ class tk_cache_desc(ctypes.Structure):
         "max_pages_per_seq", "k_dtype")]
 
 
-NATIVE_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tkpy.so")
+NATIVE_PATH = build.PY_LIB
 _NATIVE_CALLS = ("tk_kv_append", "tk_attn_decode", "tk_attn_decode_append", "tk_attn_decode_noalloc",
                  "tk_attn_prefill", "tk_attn_forward", "tk_attn_backward", "tk_attn_prefill_cached")
 
@@ -95,7 +97,6 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
-    _load_native(L)
     _lib = L
     return L
 
@@ -103,9 +104,9 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
 def _load_native(L: ctypes.CDLL):
     """Load _tkpy.so and give it the addresses of the library's entry points."""
     global _native
-    if not os.path.exists(NATIVE_PATH):
-        raise RuntimeError(f"{NATIVE_PATH} is not built; run `python -m paper_2603_04427_gb300.build` "
-                           "(or __graft_entry__.build()) first")
+    if not build.py_matches():
+        raise RuntimeError(f"{NATIVE_PATH} is not built for this Python and torch ({build.py_tag()}); run "
+                           "`python -m paper_2603_04427_gb300.build` (or __graft_entry__.build()) first")
     spec = importlib.util.spec_from_file_location(f"{__package__}._tkpy", NATIVE_PATH)
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)
@@ -115,7 +116,7 @@ def _load_native(L: ctypes.CDLL):
 
 def _fast():
     if _native is None:
-        load_library()
+        _load_native(load_library())
     return _native
 
 

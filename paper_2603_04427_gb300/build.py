@@ -2,9 +2,10 @@
 
 Each ``csrc/*.cu`` is compiled by nvcc in parallel, then linked into
 ``paper_2603_04427_gb300/libtk.so``; ``csrc/py_binding.cpp`` (the binding's
-native argument checks) is compiled by g++ beside them into ``_tkpy.so``.  The
-build is skipped when both are newer than every source and header.  Run ``python -m
-paper_2603_04427_gb300.build`` (or ``__graft_entry__.build()``).
+native argument checks) is compiled by g++ beside them into ``_tkpy.so``.  Either
+is skipped when it is newer than its sources and headers and, for ``_tkpy.so``, was
+built for this Python and torch.  Run ``python -m paper_2603_04427_gb300.build`` (or
+``__graft_entry__.build()``).
 """
 
 from __future__ import annotations
@@ -12,6 +13,7 @@ from __future__ import annotations
 import concurrent.futures as cf
 import glob
 import os
+import platform
 import shutil
 import subprocess
 import sys
@@ -25,6 +27,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtk.so")
 PY_SRC = os.path.join(CSRC, "py_binding.cpp")
 PY_LIB = os.path.join(PKG, "_tkpy.so")
+PY_TAG = os.path.join(BUILD, "_tkpy.tag")   # what _tkpy.so was built for
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
@@ -43,15 +46,46 @@ def _sources():
 
 
 def _deps():
-    return _sources() + [PY_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
-        os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(
+        os.path.join(CSRC, "*.h")) + _headers()
+
+
+def _headers():
+    return glob.glob(os.path.join(INCLUDE, "*.h"))
+
+
+def _newer(lib: str, deps) -> bool:
+    if not os.path.exists(lib):
+        return False
+    t = os.path.getmtime(lib)
+    return all(os.path.getmtime(f) <= t for f in [*deps, __file__])
+
+
+def lib_up_to_date() -> bool:
+    return _newer(LIB, _deps())
+
+
+def py_tag() -> str:
+    """What _tkpy.so depends on beside its sources: CPython's and torch's C++ interfaces."""
+    import torch
+    return (f"{sys.implementation.cache_tag} {platform.machine()} torch {torch.__version__} "
+            f"cxx11_abi {int(torch.compiled_with_cxx11_abi())}")
+
+
+def py_matches() -> bool:
+    """_tkpy.so exists and was built for this Python and torch."""
+    if not os.path.exists(PY_LIB) or not os.path.exists(PY_TAG):
+        return False
+    with open(PY_TAG) as f:
+        return f.read() == py_tag()
+
+
+def py_up_to_date() -> bool:
+    return _newer(PY_LIB, [PY_SRC] + _headers()) and py_matches()
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PY_LIB):
-        return False
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PY_LIB))
-    return all(os.path.getmtime(f) <= t for f in _deps() + [__file__])
+    return lib_up_to_date() and py_up_to_date()
 
 
 def _compile(src: str, extra) -> str:
@@ -81,26 +115,34 @@ def _build_py() -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for {PY_SRC}:\n{' '.join(cmd)}\n{r.stdout}\n{r.stderr}")
+    if os.path.exists(PY_TAG):   # no tag beside another module, whatever happens next
+        os.remove(PY_TAG)
     os.replace(tmp, PY_LIB)
+    with open(PY_TAG + ".tmp", "w") as f:
+        f.write(py_tag())
+    os.replace(PY_TAG + ".tmp", PY_TAG)
 
 
 def build(force: bool = False, verbose_ptxas: bool = False) -> str:
-    """Compile and link libtk.so; returns its path."""
-    if not force and up_to_date():
+    """Compile and link libtk.so and _tkpy.so where they are not up to date; returns libtk.so's path."""
+    want_lib, want_py = force or not lib_up_to_date(), force or not py_up_to_date()
+    if not want_lib and not want_py:
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     extra = ["-Xptxas", "-v"] if verbose_ptxas else []
-    srcs = _sources()
+    srcs = _sources() if want_lib else []
     with cf.ThreadPoolExecutor(max_workers=max(1, min(len(srcs) + 1, os.cpu_count() or 1))) as ex:
-        py = ex.submit(_build_py)
+        py = ex.submit(_build_py) if want_py else None
         objs = list(ex.map(lambda s: _compile(s, extra), srcs))
-    py.result()
-    tmp = LIB + ".tmp"
-    cmd = [nvcc()] + ARCH + ["-shared", "-o", tmp] + objs
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError(f"link failed:\n{' '.join(cmd)}\n{r.stdout}\n{r.stderr}")
-    os.replace(tmp, LIB)
+    if want_lib:
+        tmp = LIB + ".tmp"
+        cmd = [nvcc()] + ARCH + ["-shared", "-o", tmp] + objs
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"link failed:\n{' '.join(cmd)}\n{r.stdout}\n{r.stderr}")
+        os.replace(tmp, LIB)
+    if py is not None:
+        py.result()   # libtk.so, which needs no torch, stands whatever became of _tkpy.so
     return LIB
 
 

@@ -67,6 +67,21 @@ def test_host_tensors_are_left_to_the_python_checks(name):
         fn(*args)
 
 
+def test_a_module_built_for_another_torch_is_rebuilt_and_not_loaded(monkeypatch):
+    """_tkpy.so is compiled against torch's C++ tensors: after a change of torch (or of Python) it
+    counts as out of date and is refused, where its accessors could read another layout.  The C
+    library, which needs neither, still loads and is not built again."""
+    tbuild.build()
+    assert tbuild.up_to_date()
+    monkeypatch.setattr(tbuild, "py_tag", lambda: "another")
+    assert not tbuild.up_to_date() and tbuild.lib_up_to_date()
+    monkeypatch.setattr(tb, "_native", None)
+    monkeypatch.setattr(tb, "_lib", None)
+    assert tb.tk_status_string(tb.TK_OK) == "TK_OK"
+    with pytest.raises(RuntimeError, match="not built for this Python and torch"):
+        tb._fast()
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("name", NAMES)
 def test_both_routes_make_the_same_call(name, monkeypatch):
