@@ -153,13 +153,20 @@ struct Cache {
   }
 };
 
+// Holds the GIL released; takes it back however the scope is left.
+struct NoGil {
+  PyThreadState* state = PyEval_SaveThread();
+  ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 // Makes the C call without the GIL; its status as a Python int.
 template <typename F>
 PyObject* call(F&& f) {
   tk_status s;
-  Py_BEGIN_ALLOW_THREADS
-  s = f();
-  Py_END_ALLOW_THREADS
+  {
+    NoGil scope;
+    s = f();
+  }
   return PyLong_FromLong(s);
 }
 
