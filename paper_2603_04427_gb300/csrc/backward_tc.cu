@@ -303,8 +303,8 @@ __device__ __forceinline__ void sum_split(const BackwardParams& p, unsigned char
 }
 
 // SPLIT: the CTAs of a cluster share a key tile's query tiles and add up their dK
-// and dV through distributed shared memory at the end; for launches of so few key
-// tiles that SMs would stay idle (choose_split).
+// and dV through distributed shared memory at the end; for launches whose key tiles
+// are too few or too uneven to keep the SMs busy alone (backward_split).
 template <int R, int DV, bool SPLIT>
 __global__ void __launch_bounds__(kTcBound, 1)
 bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
@@ -522,7 +522,7 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
           if (h == 1) {
             // dQ before the next tile's half-1 scores: with one dS tile the next
             // tile's half-0 dS waits for it, and without columns of its own dQ
-            // occupies S^T_1 / dP^T_1 until warps 4-7 have read it
+            // occupies S^T_1 / dP^T_1 until the dQ warps have read it
             if (C::DQ_OWN && t > 0 && !(ok = wait_all(dq_empty, (t - 1) & 1))) break;
             tc_fence_after();
             issue_dq(t);
@@ -705,35 +705,6 @@ bwd_tc_kernel(const __grid_constant__ TcMaps maps, const BackwardParams p) {
   }
 }
 
-// CTAs per key tile: the number with the least estimated time, in units of one
-// tile's (1.6 us at r = 32): a CTA costs 5 for set-up and epilogue, 2 more if
-// split; causal launches (CTAs of many sizes, the largest first) take the longer of
-// their heaviest CTA and the mean of the SMs, and half a set-up more where a split
-// needs a second CTA on an SM; others whole waves.  A CTA keeps at least two of its
-// key tile's query tiles.  Measured without and with the split: 16/2 heads, r=64,
-// d_v=128, B=3, S=138 41 us -> 16; r=32, B=1, S=2000 206 -> 59; r=128, S=500 117 -> 28;
-// 32/8 heads, r=32, S=300 26 -> 16, S=1531 87 -> 53; but 12 heads, r=16, d_v=64, S=1024
-// 17.4 -> 21.1 with two CTAs a key tile (192 on 152 SMs), so that one is not split.
-int choose_split(const BackwardParams& p, long long grid) {
-  const int n_qt = (p.S + kQT - 1) / kQT;
-  const double heaviest = static_cast<double>(p.Hq / p.Hkv) * n_qt;   // the first key tile's
-  const double total = heaviest * grid * (p.causal ? (n_qt + 1) / (2.0 * n_qt) : 1.0);
-  int best = 1;
-  double least = 0;
-  for (int c = 1; c <= kMaxSplit; c *= 2) {
-    if (c > 1 && heaviest < 2 * c) break;
-    const double fixed = c > 1 ? 7 : 5, one = heaviest / c + fixed;
-    const double mean = (total + grid * c * fixed) / p.num_sms;
-    const double t = p.causal ? std::max(one, mean) + (c > 1 && grid * c > p.num_sms ? fixed / 2 : 0)
-                              : std::ceil(static_cast<double>(grid) * c / p.num_sms) * one;
-    if (c == 1 || t < 0.95 * least) {
-      best = c;
-      least = t;
-    }
-  }
-  return best;
-}
-
 template <int R, int DV>
 cudaError_t launch_tc(const BackwardParams& p, cudaStream_t stream) {
   using C = TCfg<R, DV>;
@@ -750,9 +721,8 @@ cudaError_t launch_tc(const BackwardParams& p, cudaStream_t stream) {
   const long long grid = static_cast<long long>(p.B) * p.Hkv * n_kt;
   if (grid > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   BackwardParams pp = p;
-  pp.split = choose_split(p, grid);
-  // Q and dO of all heads within about 48 MB of L2
-  pp.tile_major = static_cast<long long>(p.B) * p.Hq * p.S * (R + DV) * 2 <= (48LL << 20);
+  pp.split = backward_split(p.B, p.Hq, p.Hkv, p.S, p.causal != 0, p.num_sms);
+  pp.tile_major = backward_tile_major(p.B, p.Hq, p.S, R, DV);
   auto kern = pp.split > 1 ? bwd_tc_kernel<R, DV, true> : bwd_tc_kernel<R, DV, false>;
   const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;

@@ -14,6 +14,12 @@ extern "C" int prefill_shares(long long kv_tiles, int most) { return tk::prefill
 extern "C" int prefill_cluster(long long pairs, long long kv_tiles, int num_sms) {
   return tk::prefill_cluster(pairs, kv_tiles, num_sms);
 }
+extern "C" int backward_split(int batch, int h_q, int h_kv, int seq, int causal, int num_sms) {
+  return tk::backward_split(batch, h_q, h_kv, seq, causal != 0, num_sms);
+}
+extern "C" int backward_tile_major(int batch, int h_q, int seq, int r, int d_v) {
+  return tk::backward_tile_major(batch, h_q, seq, r, d_v);
+}
 """
 
 
@@ -28,6 +34,11 @@ def rules():
     L.prefill_shares.argtypes = [ctypes.c_longlong, ctypes.c_int]
     L.prefill_cluster.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
     return L
+
+
+def sms():
+    import torch
+    return torch.cuda.get_device_properties(0).multi_processor_count
 
 
 def tiles(n):

@@ -6,7 +6,8 @@ distributed shared memory.  Covered:
 every split, shares without a tile for query tile A or for any (causal pairs
 early in the sequence), rows that a share sees nothing of (contexts that end
 off a tile boundary), every output type, key format, r / d_v staging layout,
-and that a sequence's result does not depend on the split beyond rounding.
+and that the result is the unsplit kernel's (tk_attn_forward's) but for the
+rounding of the softmax weights.  The split of each case (on 152 SMs) is asserted.
 """
 
 import math
@@ -15,7 +16,7 @@ import pytest
 import torch
 
 from _helpers import f64, parity, parity_bf16, require_gpu
-from _split import prefill_pairs, rules, tiles
+from _split import prefill_pairs, rules, sms, tiles
 from oracle import attention as oa
 from oracle import cache as oc
 from paper_2603_04427_gb300 import binding as tb
@@ -24,16 +25,22 @@ from paper_2603_04427_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B,hq,hkv,S,r,dv,bf16,causal", [
-    (1, 4, 4, 1281, 32, 128, False, True),    # 24 pairs, 11 kv tiles: split 2
-    (1, 2, 1, 1700, 16, 64, True, True),      # 14 kv tiles: split 4
-    (1, 1, 1, 3100, 64, 128, False, True),    # 25 kv tiles: split 8
-    (1, 1, 1, 4097, 32, 128, True, True),     # 33 kv tiles: split 8
-    (1, 2, 2, 1300, 128, 128, False, False),  # full attention
-    (1, 1, 1, 1921, 128, 64, False, False),   # a last pair of one row
-])
-def test_prefill_split(B, hq, hkv, S, r, dv, bf16, causal):
+def _assert_split(B, hq, S, tokens, split):
     require_gpu()
+    if sms() == 152:
+        assert rules().prefill_cluster(prefill_pairs(B, hq, S), tiles(tokens), 152) == split
+
+
+@pytest.mark.parametrize("B,hq,hkv,S,r,dv,bf16,causal,split", [
+    (1, 4, 4, 1281, 32, 128, False, True, 2),    # 24 pairs, 11 kv tiles
+    (1, 2, 1, 1700, 16, 64, True, True, 4),      # 14 kv tiles
+    (1, 1, 1, 3100, 64, 128, False, True, 8),    # 25 kv tiles
+    (1, 1, 1, 4097, 32, 128, True, True, 8),     # 33 kv tiles
+    (1, 2, 2, 1300, 128, 128, False, False, 2),  # full attention
+    (1, 1, 1, 1921, 128, 64, False, False, 4),   # a last query tile of one row
+])
+def test_prefill_split(B, hq, hkv, S, r, dv, bf16, causal, split):
+    _assert_split(B, hq, S, S, split)
     q = inputs.normal_bf16((B, hq, S, r), 91, device="cuda")
     k = inputs.normal_bf16((B, hkv, S, r), 92, device="cuda")
     v = inputs.normal_bf16((B, hkv, S, dv), 93, device="cuda")
@@ -42,17 +49,20 @@ def test_prefill_split(B, hq, hkv, S, r, dv, bf16, causal):
     assert tb.tk_get_device_error() == 0
     ref = oa.attention_prefill(f64(q), f64(k), f64(v), 1 / math.sqrt(r), causal=causal)
     (parity_bf16 if bf16 else parity)(f64(out), ref, what=f"split prefill S={S} r={r} d_v={dv}")
+    whole, lse = torch.empty((B, hq, S, dv), device="cuda"), torch.empty((B, hq, S), device="cuda")
+    tb.tk_attn_forward(q, k, v, whole, lse, causal=causal)
+    (parity_bf16 if bf16 else parity)(f64(out), f64(whole), what=f"split against unsplit S={S} r={r} d_v={dv}")
 
 
-@pytest.mark.parametrize("hq,hkv,S,lens,r,dv,page,keys", [
-    (4, 2, 23, [3001, 1], 32, 128, 0, "bf16"),     # one query tile, split 8 and mostly empty shares
-    (4, 1, 130, [2000, 777], 64, 64, 16, "bf16"),  # two tiles, the second of two rows
-    (2, 2, 300, [1111], 32, 128, 64, "int8"),      # hi + lo keys
-    (2, 1, 200, [1500], 128, 128, 0, "int4"),      # scales in the softmax
-    (8, 2, 256, [130, 1200], 16, 128, 128, "bf16"),
+@pytest.mark.parametrize("hq,hkv,S,lens,r,dv,page,keys,split", [
+    (4, 2, 23, [3001, 1], 32, 128, 0, "bf16", 8),     # one query tile; the second sequence not split
+    (4, 1, 130, [2000, 777], 64, 64, 16, "bf16", 4),  # two tiles, the second of two rows
+    (2, 2, 300, [1111], 32, 128, 64, "int8", 4),      # hi + lo keys
+    (2, 1, 200, [1500], 128, 128, 0, "int4", 4),      # scales in the softmax
+    (8, 2, 256, [130, 1200], 16, 128, 128, "bf16", 4),
 ])
-def test_chunk_split(hq, hkv, S, lens, r, dv, page, keys):
-    require_gpu()
+def test_chunk_split(hq, hkv, S, lens, r, dv, page, keys, split):
+    _assert_split(len(lens), hq, S, max(lens) + S, split)
     B, L = len(lens), max(lens) + S
     cap = (L + 15) // 16 * 16
     kw = dict(k_int8=keys == "int8", k_int4=keys == "int4")
@@ -138,11 +148,9 @@ def test_the_bound_does_not_change_the_result(B, hq, hkv, S, lens, r, dv, page, 
     """A loose max_seq_len launches clusters of up to eight CTAs over short contexts: each
     sequence is split by its own length, so the bits are those of a tight bound (and, for an
     empty cache, of the plain prefill)."""
-    require_gpu()
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
     tight, loose = max(lens) + S, 16384
-    own = rules().prefill_cluster(prefill_pairs(B, hq, S), tiles(tight), sms)
-    assert own == shares and rules().prefill_cluster(prefill_pairs(B, hq, S), tiles(loose), sms) > min(shares, 4)
+    _assert_split(B, hq, S, tight, shares)
+    _assert_split(B, hq, S, loose, 8)
     g = dict(device="cuda")
     kw = dict(k_int8=keys == "int8", k_int4=keys == "int4")
     if page:

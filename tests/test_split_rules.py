@@ -1,6 +1,6 @@
 """The rules that split work over a cluster's CTAs (csrc/split.h), on the CPU."""
 
-from _split import rules
+from _split import rules, tiles
 
 
 def test_a_sequences_shares_do_not_depend_on_the_launch_bound():
@@ -25,3 +25,16 @@ def test_prefill_clusters_fit_the_sms_and_every_size_occurs():
             seen.add(n)
             assert n == 1 or (pairs * n <= 152 and tiles >= 10 and tiles // n >= 3)
     assert seen == {1, 2, 4, 8}
+
+
+def test_backward_splits_keep_work_for_the_heaviest_tiles_ctas():
+    R = rules()
+    seen = set()
+    for B, hq, hkv in ((1, 1, 1), (1, 8, 1), (2, 16, 2), (1, 32, 8), (8, 12, 12), (4, 16, 16)):
+        for S in (1, 100, 129, 300, 528, 1000, 1921, 4096):
+            for causal in (0, 1):
+                n = R.backward_split(B, hq, hkv, S, causal, 152)
+                seen.add(n)
+                assert n == 1 or hq // hkv * tiles(S) >= 2 * n
+    assert seen == {1, 2, 4, 8}
+    assert R.backward_split(1, 12, 12, 1024, 1, 152) == 1   # measured: two CTAs a key tile are slower
