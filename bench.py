@@ -922,7 +922,7 @@ def main():
                                  "peak_source": peak_src,
                                  "traffic": recorded_traffic("prefill", pw.name, source_hash(
                                      "prefill.cu", "common.cuh", "tc05.cuh", "widen.cuh",
-                                     "kernels.h"))})
+                                     "kernels.h", "split.h"))})
         else:
             pre.update(pf)
         if n == 1:

@@ -39,6 +39,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -56,6 +57,7 @@ constexpr int kLenMask = 0x7fffffff;        // a context length; the sign bit ma
 constexpr int kMaxSub = 4;                  // pages of 16 tokens in one unit
 constexpr int kMaxBatch = 1024;             // prefix arrays live in shared memory
 constexpr int kCtaSmemTarget = 110 * 1024;  // aim for two CTAs per SM
+constexpr int kLongStream = 192;            // chunks per CTA from which a stream is long
 
 // KF: key format, 0 bf16, 1 int8, 2 int4 (two codes per byte, R >= 32).
 template <int R, int DV, int G, int KF>
@@ -83,8 +85,24 @@ struct Cfg {
   // two CTAs per SM when at least three stages fit in half the SM
   static constexpr int CTAS_PER_SM = NSTAGE_2 >= 3 ? 2 : 1;
   static constexpr int NSTAGE_RAW = CTAS_PER_SM == 2 ? NSTAGE_2 : NSTAGE_1;
-  static constexpr int NSTAGE = NSTAGE_RAW > 8 ? 8 : NSTAGE_RAW;
+  // Bytes on their way to an SM.  More than about 160 KB are of no use, and in long
+  // streams of chunks of 16 KB and more 100 to 130 KB are best: the memory is busy
+  // either way, and deeper rings only scatter its accesses.  Short streams want the
+  // deeper ring.  Measured, B=64, 8 kv heads, 12000 tokens (316 chunks a CTA), d_v=128,
+  // a stage less: r=128 bf16, one head 470 -> 445 -> 434 us (6, 5, 4 stages), r=32 bf16
+  // 285 -> 275, int8 262 -> 257; but B=16, 4094 tokens (27 a CTA), r=32 int8, four heads
+  // 26.2 -> 26.9.
+  static constexpr int CHUNK_BYTES = KB + VB + SB;
+  static constexpr int IN_FLIGHT_MAX = 163 * 1024 / (CTAS_PER_SM * CHUNK_BYTES);
+  static constexpr int NSTAGE = std::min({NSTAGE_RAW, IN_FLIGHT_MAX, 8});
   static_assert(NSTAGE >= 2, "shared memory budget too small for two stages");
+  // (not with eight heads or int4 keys: there the warps' work on a chunk sets the pace)
+  static constexpr bool SHALLOW = G < 8 && KF != 2 && CHUNK_BYTES >= 16 * 1024 &&
+                                  CTAS_PER_SM * (NSTAGE - 1) * CHUNK_BYTES >= 100 * 1024;
+  static constexpr int NSTAGE_LONG = SHALLOW ? NSTAGE - 1 : NSTAGE;   // for kLongStream chunks a CTA
+  // chunks of a CTA prefetched into L2 while the previous kernel finishes: twice the
+  // ring, but no more than 256 KB (B=19, 16/8 heads, 1000 tokens, r=128: 15.5 -> 14.9 us)
+  static constexpr int PREFETCH = std::min(2 * NSTAGE, 256 * 1024 / CHUNK_BYTES);
   static constexpr int RING = NSTAGE * STAGE;
   static constexpr int OFF_MERGE = RING;                         // [2][kCW][REC] f32
   static constexpr int OFF_BAR = OFF_MERGE + 2 * kCW * REC * 4;  // mbarriers
@@ -606,7 +624,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
   if (p.page_size == 0) limit = min(limit, p.capacity);
   else limit = min(limit, p.max_pages * p.page_size);
   // before the wait only reads that may be stale and L2 prefetches are issued
-  if (warp == kCW && B <= 32) prefetch_first_chunks<C::RB, DV>(p, lane, limit, 2 * C::NSTAGE);
+  if (warp == kCW && B <= 32) prefetch_first_chunks<C::RB, DV>(p, lane, limit, C::PREFETCH);
   pdl_wait();
   pdl_trigger();
 
@@ -643,6 +661,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
   // nothing.
   const Split sp(T, gridDim.x);
   const long long u_begin = c < sp.N ? sp.begin(c) : T, u_end = c < sp.N ? sp.begin(c + 1) : T;
+  const int stages = C::SHALLOW && sp.q >= kLongStream ? C::NSTAGE_LONG : C::NSTAGE;  // of the ring, in use
   // Boxes of a chunk: 64 rows, or one per page of 16 or 32 tokens.  A box holds
   // its rows' 128-byte column blocks one after the other.
   const int rows_per_box = (p.page_size == 0 || p.page_size >= kChunk) ? kChunk : p.page_size;
@@ -738,8 +757,8 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
         if (!ok) break;
         unsigned char* sk = smem + st * C::STAGE;
         if (lane == 0) {
-          // (a shift: a division here, one per chunk in the producer's chain, cost 60 cycles of a
-          // chunk's 1200; B=12, 16/8 heads, 9000 tokens, r=16, d_v=64: 30.6 -> 27.9 us a step)
+          // (a shift: a division here, one per chunk in the producer's chain, cost 120 cycles of
+          // a chunk's 1400; B=12, 16/8 heads, 9000 tokens, r=16, d_v=64: 30.6 -> 27.9 us a step)
           const int boxes = (nj + rows_per_box - 1) >> box_shift;  // nj >= 1
           mbar_arrive_expect_tx(&full[st],
                                 boxes * rows_per_box * ((C::KB + C::VB) / kChunk) + (KI8 ? ((nj + 3) & ~3) * 4 : 0) +
@@ -756,7 +775,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
           }
           if (qj >= 0) bulk_g2s(sk + C::OFF_QS, qbase + static_cast<long long>(qj) * 2, C::QB, &full[st]);
         }
-        if (++st == C::NSTAGE) {
+        if (++st == stages) {
           st = 0;
           ++use;
         }
@@ -979,7 +998,7 @@ decode_kernel(const __grid_constant__ DecodeMaps maps, const DecodeParams p) {
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[st]);
-    if (++st == C::NSTAGE) {
+    if (++st == stages) {
       st = 0;
       ph ^= 1u;
     }
