@@ -590,16 +590,23 @@ prefill_kernel(const __grid_constant__ Maps maps, const PrefillParams p) {
     const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + x * 128, tO = tmem + 256 + x * 128;
     const int row = qt * kBM + (tid & 127);    // query row of this thread in the chunk
-    const int pos = L0 + row;                  // its position among the keys
+    // Positions among the keys; in a cluster's kernel from kv tile j0 on, where this
+    // CTA's keys begin.
+    int L0x = L0, end = kv_len;
+    if constexpr (SPLIT) {
+      L0x -= j0 * kBN;
+      end -= j0 * kBN;
+    }
+    const int pos = L0x + row;                 // of this thread's row
     const float sl2 = p.scale_log2;
     float m_used = -INFINITY, l = 0.f;
     bool ok = nx > 0;
     for (int j = 0; j < nx; ++j) {
       if (!(ok = mbar_wait_warp(&s_full[x], j & 1, p.err))) break;
       tc_fence_after();
-      const int kv0 = (j0 + j) * kBN;
-      const bool masked = (p.causal && kv0 + kBN - 1 > L0 + qt * kBM) || (kv0 + kBN > kv_len);
-      const int lim = min(kv_len - kv0, p.causal ? pos - kv0 + 1 : kBN);  // visible columns
+      const int kv0 = j * kBN;
+      const bool masked = (p.causal && kv0 + kBN - 1 > L0x + qt * kBM) || (kv0 + kBN > end);
+      const int lim = min(end - kv0, p.causal ? pos - kv0 + 1 : kBN);  // visible columns
       // the whole S row of this thread: 128 fp32 scores
       uint32_t v[128];
       tmem_ld128(tS + lane_off, v);
